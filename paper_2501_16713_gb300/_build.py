@@ -34,9 +34,16 @@ SOURCES = [
     "fista.cu",
     "motion.cu",
     "fft_pruned.cu",
+    "fft_mixed.cu",
+    "fft_mixed_static.cu",
+    "fft_mixed_rt_coil.cu",
+    "fft_mixed_rt_image.cu",
+    "fft_mixed_gen_coil.cu",
+    "fft_mixed_gen_image.cu",
     "spread_home.cu",
 ]
-HEADERS = ["common.cuh", "plan_internal.h", "kb_host.h"]
+HEADERS = ["common.cuh", "plan_internal.h", "kb_host.h", "fft_mixed.cuh",
+           "fft_mixed_kernels.cuh"]
 
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 

@@ -205,6 +205,30 @@ nrsense_status image_grid_adjoint(nrsense_plan_s* p, nrsense_c64* xhat, cudaStre
   return launched();
 }
 
+// u (b_ugrid) = F_G^-1 Z (1/C) F_N x, the upsampled image of T, and its adjoint
+nrsense_status image_up(nrsense_plan_s* p, const nrsense_c64* x, cudaStream_t s) {
+  if (p->image_mixed && p->own_image_fft()) {
+    STAGE(FFT_G, launch_mixed_image_up(p->geo, p->mix, p->deapod, x, p->b_ugrid, p->b_upad,
+                                       p->b_ugrid, s));
+    p->upad_dirty = true;
+    return launched();
+  }
+  NRS_TRY(fft(p, NRSENSE_STAGE_FFT_N, p->fft_n, s, const_cast<nrsense_c64*>(x), p->b_xhat,
+              CUFFT_FORWARD));
+  return image_grid_forward(p, s);
+}
+
+nrsense_status image_down(nrsense_plan_s* p, nrsense_c64* x, cudaStream_t s) {
+  if (p->image_mixed && p->own_image_fft()) {
+    STAGE(FFT_G, launch_mixed_image_down(p->geo, p->mix, p->deapod, p->b_ugrid, p->b_upad,
+                                         p->b_ugrid, x, s));
+    p->upad_dirty = true;
+    return launched();
+  }
+  NRS_TRY(image_grid_adjoint(p, x, s));
+  return fft(p, NRSENSE_STAGE_FFT_N, p->fft_n, s, x, x, CUFFT_INVERSE);
+}
+
 // m (P x nvox) = T_j x for all phases
 nrsense_status warp_forward(nrsense_plan_s* p, const nrsense_c64* x, nrsense_c64* m,
                             cudaStream_t s) {
@@ -213,8 +237,7 @@ nrsense_status warp_forward(nrsense_plan_s* p, const nrsense_c64* x, nrsense_c64
     STAGE(VECTOR, launch_copy_phases(g, p->P, x, m, s));
     return launched();
   }
-  NRS_TRY(fft(p, NRSENSE_STAGE_FFT_N, p->fft_n, s, const_cast<nrsense_c64*>(x), p->b_xhat, CUFFT_FORWARD));
-  NRS_TRY(image_grid_forward(p, s));
+  NRS_TRY(image_up(p, x, s));
   if (p->interp_home && p->home_ok) {
     STAGE(INTERP_IMAGE, launch_interp_home(g, p->kc, p->ihome, p->b_ugrid, m, s));
   } else {
@@ -240,8 +263,7 @@ nrsense_status warp_adjoint(nrsense_plan_s* p, const nrsense_c64* m, nrsense_c64
                                       p->d_status, s));
   }
   NRS_TRY(launched());
-  NRS_TRY(image_grid_adjoint(p, x, s));
-  return fft(p, NRSENSE_STAGE_FFT_N, p->fft_n, s, x, x, CUFFT_INVERSE);
+  return image_down(p, x, s);
 }
 
 // The cuFFT forward path reads the zero padding of b_xpad and b_xmid; the
@@ -262,9 +284,13 @@ nrsense_status sense_chunk_forward(nrsense_plan_s* p, int j0, int j1, const nrse
                                    nrsense_c64* y, long long row_base, cudaStream_t s) {
   const Geo& g = p->geo;
   const int nph = j1 - j0;
-  if (p->fft_pruned) {
-    STAGE(FFT_PRUNED, launch_pruned_forward(g, p->C, nph, p->kcolmask, p->deapod, p->smaps, m, p->b_xpad,
-                                            p->b_xmid, p->b_xwork, s));
+  if (p->own_fft()) {
+    STAGE(FFT_PRUNED,
+          p->coil_mixed
+              ? launch_mixed_forward(g, p->mix, p->C, nph, p->kcolmask, p->kanymask, p->deapod,
+                                     p->smaps, m, p->b_xpad, p->b_xmid, p->b_xwork, s)
+              : launch_pruned_forward(g, p->C, nph, p->kcolmask, p->kanymask, p->deapod, p->smaps, m,
+                                      p->b_xpad, p->b_xmid, p->b_xwork, s));
     p->pad_dirty = true;
     NRS_TRY(launched());
   } else {
@@ -290,9 +316,13 @@ nrsense_status sense_chunk_adjoint(nrsense_plan_s* p, int j0, int j1, const nrse
   STAGE(SPREAD_KSPACE, launch_spread(g, p->W, p->kc, p->C, p->ktiles, t, y, p->b_xspread,
                                      p->grid_bf16, p->comp_spread, p->spread_variant, p->b_scratch, p->d_status, s));
   NRS_TRY(launched());
-  if (p->fft_pruned) {
-    STAGE(FFT_PRUNED, launch_pruned_inverse(g, p->C, nph, p->kcolmask, p->deapod, p->smaps, p->b_xspread,
-                                            p->b_xmid, p->b_xpad, w, s));
+  if (p->own_fft()) {
+    STAGE(FFT_PRUNED,
+          p->coil_mixed
+              ? launch_mixed_inverse(g, p->mix, p->C, nph, p->kcolmask, p->kanymask, p->deapod,
+                                     p->smaps, p->b_xspread, p->b_xmid, p->b_xpad, w, s)
+              : launch_pruned_inverse(g, p->C, nph, p->kcolmask, p->kanymask, p->deapod, p->smaps,
+                                      p->b_xspread, p->b_xmid, p->b_xpad, w, s));
     p->pad_dirty = true;
     return launched();
   }
@@ -526,14 +556,14 @@ nrsense_status nrsense_plan_autotune(nrsense_plan_t p, int32_t reps, nrsense_tun
     p->interp_home = out->interp_image_ms[1] >= 0.0 &&
                      out->interp_image_ms[1] < out->interp_image_ms[0];
     out->interp_image_home = p->interp_home ? 1 : 0;
-    // image-space G^3 transforms with their deapodization, forward and
-    // adjoint: cuFFT path vs the pruned passes (inputs: the plan's buffers)
+    // image-space N^3 and G^3 transforms with their deapodization, forward and
+    // adjoint: cuFFT path vs the own passes (inputs: the plan's buffers)
     for (int k = 0; k < 2 && p->image_fft_ok; ++k) {
       p->image_fft_pruned = k == 1;
       nrsense_status st = NRSENSE_OK;
       auto run = [&] {
-        if (st == NRSENSE_OK) st = image_grid_forward(p, s);
-        if (st == NRSENSE_OK) st = image_grid_adjoint(p, p->b_tmp, s);
+        if (st == NRSENSE_OK) st = image_up(p, p->b_m, s);
+        if (st == NRSENSE_OK) st = image_down(p, p->b_tmp, s);
       };
       run();
       cudaEventRecord(a, s);

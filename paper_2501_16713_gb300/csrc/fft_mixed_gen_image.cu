@@ -1,0 +1,15 @@
+// The mixed-radix image-space passes (fft_mixed_kernels.cuh) for axes of any
+// oversampling factor and length: two- or three-step transforms with run-time
+// radices (a translation unit of its own: one unrolled body per radix).
+#include "fft_mixed_kernels.cuh"
+
+namespace nrs {
+
+void mixed_gen_image_pass(const MixPass& a, const MixAxis& x, cudaStream_t s) {
+  mixed::GeneralAxis ax{x.g, x.n, x.N};
+  ax.g.tw = x.tw_g;
+  ax.n.tw = x.tw_n;
+  mixed::run_image_pass(a, ax, s);
+}
+
+}  // namespace nrs

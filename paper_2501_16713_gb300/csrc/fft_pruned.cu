@@ -261,15 +261,24 @@ __global__ void __launch_bounds__(Shape<R1, R2>::threads, 4) fwd_x_kernel(
 }
 
 // F2: T2[slot][i0][:][x] = DFT_y of T1[slot][i0][data rows][x] (exponent sign
-// + for INV).
+// + for INV).  anymask (or null): per x tile a bit per y tile whose tile column
+// has a tile of the union; the z passes skip the other columns, so they are
+// neither stored here nor loaded by I2 (sense128: 15 % of T2's traffic).
 // CTA: (block of 16 x, i0, slot).
 template <int R1, int R2, bool INV>
 __global__ void __launch_bounds__(Shape<R1, R2>::threads, 5) fwd_y_kernel(
-    PassGeo g, const float2* __restrict__ t1, float2* __restrict__ t2) {
+    PassGeo g, const uint32_t* __restrict__ anymask, const float2* __restrict__ t1,
+    float2* __restrict__ t2) {
   __shared__ float2 sy[Shape<R1, R2>::smem];
   __shared__ float2 tw[R1 * R2];
-  fill_twiddles<R1 * R2>(tw);
   const int xb = blockIdx.x, i0 = blockIdx.y;
+  uint32_t m0 = ~0u, m1 = ~0u;
+  if (anymask != nullptr) {
+    m0 = __ldg(anymask + 2 * xb);
+    m1 = __ldg(anymask + 2 * xb + 1);
+    if ((m0 | m1) == 0u) return;  // CTA-uniform
+  }
+  fill_twiddles<R1 * R2>(tw);
   const long long slot = blockIdx.z;
   const float2* src = t1 + (slot * g.n0 + i0) * g.n1 * (long long)g.g2;
   float2* dst = t2 + (slot * g.n0 + i0) * g.g1 * (long long)g.g2;
@@ -278,7 +287,8 @@ __global__ void __launch_bounds__(Shape<R1, R2>::threads, 5) fwd_y_kernel(
   };
   auto st = [&](int col, int k1, auto k2c, float2 v) {
     constexpr int k2 = decltype(k2c)::value;
-    dst[(k1 + R1 * k2) * g.g2 + xb * kCols + col] = v;
+    const int y = k1 + R1 * k2;
+    if (((col < 8 ? m0 : m1) >> (y >> 3)) & 1u) dst[y * g.g2 + xb * kCols + col] = v;
   };
   fft16<R1, R2, INV, false, true, false>(sy, tw, ld, st);
 }
@@ -326,14 +336,15 @@ __global__ void __launch_bounds__(Shape<R1, R2>::threads, 5) inv_z_kernel(
     float2* __restrict__ t2) {
   __shared__ float2 sy[Shape<R1, R2>::smem];
   __shared__ float2 tw[R1 * R2];
-  fill_twiddles<R1 * R2>(tw);
   const int xb = blockIdx.x, y = blockIdx.y;
   uint32_t m0 = ~0u, m1 = ~0u;
   if (colmask != nullptr) {
     const uint32_t* cm = colmask + (y >> 3) * (g.g2 >> 3) + 2 * xb;
     m0 = __ldg(cm);
     m1 = __ldg(cm + 1);
+    if ((m0 | m1) == 0u) return;  // CTA-uniform; I2 does not read these columns
   }
+  fill_twiddles<R1 * R2>(tw);
   const long long slot = blockIdx.z;
   const long long plane = (long long)g.g1 * g.g2;
   const float2* src = grid + slot * g.g0 * plane + (long long)y * g.g2 + xb * kCols;
@@ -354,16 +365,24 @@ __global__ void __launch_bounds__(Shape<R1, R2>::threads, 5) inv_z_kernel(
 // data rows.
 template <int R1, int R2, bool INV>
 __global__ void __launch_bounds__(Shape<R1, R2>::threads, 5) inv_y_kernel(
-    PassGeo g, const float2* __restrict__ t2, float2* __restrict__ t1) {
+    PassGeo g, const uint32_t* __restrict__ anymask, const float2* __restrict__ t2,
+    float2* __restrict__ t1) {
   __shared__ float2 sy[Shape<R1, R2>::smem];
   __shared__ float2 tw[R1 * R2];
   fill_twiddles<R1 * R2>(tw);
   const int xb = blockIdx.x, i0 = blockIdx.y;
+  uint32_t m0 = ~0u, m1 = ~0u;
+  if (anymask != nullptr) {
+    m0 = __ldg(anymask + 2 * xb);
+    m1 = __ldg(anymask + 2 * xb + 1);
+  }
   const long long slot = blockIdx.z;
   const float2* src = t2 + (slot * g.n0 + i0) * g.g1 * (long long)g.g2;
   float2* dst = t1 + (slot * g.n0 + i0) * g.n1 * (long long)g.g2;
   auto ld = [&](int col, int n1, int t) -> float2 {
-    return src[(R2 * n1 + t) * g.g2 + xb * kCols + col];
+    const int y = R2 * n1 + t;
+    return (((col < 8 ? m0 : m1) >> (y >> 3)) & 1u) ? src[y * g.g2 + xb * kCols + col]
+                                                    : make_float2(0.f, 0.f);
   };
   auto st = [&](int col, int k1, auto k2c, float2 v) {
     constexpr int k2 = decltype(k2c)::value;
@@ -544,7 +563,7 @@ bool pruned_image_fft_supported(const Geo& g) {
 cudaError_t init_pruned_fft() { return cudaSuccess; }  // no tables to upload
 
 int launch_pruned_forward(const Geo& g, int C, int nph, const uint32_t* colmask,
-                          const float* deapod,
+                          const uint32_t* anymask, const float* deapod,
                           const nrsense_c64* smaps, const nrsense_c64* m, void* t1, void* t2,
                           void* grid, cudaStream_t s) {
   const PassGeo pg = pass_geo(g, C, nph);
@@ -554,14 +573,14 @@ int launch_pruned_forward(const Geo& g, int C, int nph, const uint32_t* colmask,
   const unsigned slots = unsigned(C * nph);
   NRS_LAUNCH_L(fwd_x_kernel, g.g2, dim3((g.n1 + kCols - 1) / kCols, g.n0, nph), s, pg, deapod,
                reinterpret_cast<const float2*>(smaps), reinterpret_cast<const float2*>(m), T1);
-  NRS_LAUNCH_LS(fwd_y_kernel, false, g.g1, dim3(g.g2 / kCols, g.n0, slots), s, pg, T1, T2);
+  NRS_LAUNCH_LS(fwd_y_kernel, false, g.g1, dim3(g.g2 / kCols, g.n0, slots), s, pg, anymask, T1, T2);
   NRS_LAUNCH_LS(fwd_z_kernel, false, g.g0, dim3(g.g2 / kCols, g.g1, slots), s, pg, colmask, T2,
                 Gd);
   return 3;
 }
 
 int launch_pruned_inverse(const Geo& g, int C, int nph, const uint32_t* colmask,
-                          const float* deapod,
+                          const uint32_t* anymask, const float* deapod,
                           const nrsense_c64* smaps, const void* grid, void* t2, void* t1,
                           nrsense_c64* w, cudaStream_t s) {
   const PassGeo pg = pass_geo(g, C, nph);
@@ -571,7 +590,7 @@ int launch_pruned_inverse(const Geo& g, int C, int nph, const uint32_t* colmask,
   const unsigned slots = unsigned(C * nph);
   NRS_LAUNCH_LS(inv_z_kernel, true, g.g0, dim3(g.g2 / kCols, g.g1, slots), s, pg, colmask, Gd,
                 T2);
-  NRS_LAUNCH_LS(inv_y_kernel, true, g.g1, dim3(g.g2 / kCols, g.n0, slots), s, pg, T2, T1);
+  NRS_LAUNCH_LS(inv_y_kernel, true, g.g1, dim3(g.g2 / kCols, g.n0, slots), s, pg, anymask, T2, T1);
   NRS_LAUNCH_L(inv_x_kernel, g.g2, dim3((g.n1 + kCols - 1) / kCols, g.n0, nph), s, pg, deapod,
                reinterpret_cast<const float2*>(smaps), T1, reinterpret_cast<float2*>(w));
   return 3;
@@ -587,7 +606,7 @@ int launch_pruned_image_forward(const Geo& g, const float* deapod, const nrsense
   const float scale = float(1.0 / double(g.nvox));
   NRS_LAUNCH_L(timg_fwd_x_kernel, g.g2, dim3((g.n1 + kCols - 1) / kCols, g.n0, 1), s, pg, deapod,
                scale, reinterpret_cast<const float2*>(xhat), T1);
-  NRS_LAUNCH_LS(fwd_y_kernel, true, g.g1, dim3(g.g2 / kCols, g.n0, 1), s, pg, T1, T2);
+  NRS_LAUNCH_LS(fwd_y_kernel, true, g.g1, dim3(g.g2 / kCols, g.n0, 1), s, pg, nullptr, T1, T2);
   NRS_LAUNCH_LS(fwd_z_kernel, true, g.g0, dim3(g.g2 / kCols, g.g1, 1), s, pg, nullptr, T2,
                 reinterpret_cast<float2*>(ugrid));
   return 3;
@@ -602,7 +621,7 @@ int launch_pruned_image_adjoint(const Geo& g, const float* deapod, const nrsense
   const float scale = float(1.0 / double(g.nvox));
   NRS_LAUNCH_LS(inv_z_kernel, false, g.g0, dim3(g.g2 / kCols, g.g1, 1), s, pg, nullptr,
                 reinterpret_cast<const float2*>(ugrid), T2);
-  NRS_LAUNCH_LS(inv_y_kernel, false, g.g1, dim3(g.g2 / kCols, g.n0, 1), s, pg, T2, T1);
+  NRS_LAUNCH_LS(inv_y_kernel, false, g.g1, dim3(g.g2 / kCols, g.n0, 1), s, pg, nullptr, T2, T1);
   NRS_LAUNCH_L(timg_inv_x_kernel, g.g2, dim3((g.n1 + kCols - 1) / kCols, g.n0, 1), s, pg, deapod,
                scale, T1, reinterpret_cast<float2*>(xhat));
   return 3;

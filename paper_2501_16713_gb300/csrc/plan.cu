@@ -521,6 +521,40 @@ nrsense_status cufft_check(cufftResult r) {
   return r == CUFFT_SUCCESS ? NRSENSE_OK : NRSENSE_ERR_CUFFT;
 }
 
+// Radices and twiddle tables of the mixed-radix passes, where every axis has
+// them.  Compensated and BF16-storage plans keep the cuFFT path: the one asks
+// for its accuracy, the other rounds its coil grids to 8 bits, where any change
+// of the last FP32 bit before it moves results by a BF16 step.
+nrsense_status create_mixed(nrsense_plan_s* p, cudaStream_t s) {
+  const Geo& g = p->geo;
+  const int gs[3] = {g.g0, g.g1, g.g2}, ns[3] = {g.n0, g.n1, g.n2};
+  if (p->comp_spread || p->grid_bf16) return NRSENSE_OK;
+  MixAxis ax[3];
+  for (int a = 0; a < 3; ++a)
+    if (!mix_axis(ns[a], gs[a], &ax[a])) return NRSENSE_OK;
+  if (mixed_max_smem(ax) > kMixedMaxSmem) return NRSENSE_OK;
+  std::vector<float2> tw;
+  for (int k = 0; k < 6; ++k) {
+    const int L = k < 3 ? gs[k] : ns[k - 3];
+    for (int j = 0; j < L; ++j)
+      tw.push_back(make_float2(float(std::cos(2.0 * M_PI * j / L)), float(-std::sin(2.0 * M_PI * j / L))));
+  }
+  float2* d = nullptr;
+  NRS_TRY(dev_alloc_n(p, &d, (long long)tw.size()));
+  NRS_TRY(upload(d, tw, s));
+  const float2* dn = d + gs[0] + gs[1] + gs[2];
+  for (int a = 0; a < 3; ++a) {
+    ax[a].tw_g = d;
+    ax[a].tw_n = dn;
+    d += gs[a];
+    dn += ns[a];
+    p->mix[a] = ax[a];
+  }
+  if (configure_mixed(g, p->mix) != cudaSuccess) return NRSENSE_ERR_CUDA;
+  p->image_mixed = !p->identity_warp;
+  return NRSENSE_OK;
+}
+
 nrsense_status create_impl(nrsense_plan_s* p, const nrsense_desc* desc, const int64_t* n_samples,
                            const float* coords, const float* disp, const nrsense_c64* smaps,
                            cudaStream_t s) {
@@ -693,18 +727,29 @@ nrsense_status create_impl(nrsense_plan_s* p, const nrsense_desc* desc, const in
     p->kuni_fraction = double(nuni) / double(uni.size());
     // per (y, x) tile column, a bit per z tile of the union: the pruned
     // transforms store (forward) and load (adjoint) only those tiles
-    if (ktiles.nt0 <= 32) {
-      std::vector<uint32_t> cm((size_t)ktiles.nt1 * ktiles.nt2, 0u);
-      long long ncol = 0;
+    {
+      const size_t cols = (size_t)ktiles.nt1 * ktiles.nt2;
+      std::vector<uint32_t> cm(cols * ((ktiles.nt0 + 31) / 32), 0u);
+      std::vector<char> any(cols, 0);
       for (long long t = 0; t < ktiles.ntiles; ++t)
         if (uni[(size_t)t]) {
-          const long long col = t % ((long long)ktiles.nt1 * ktiles.nt2);
-          cm[(size_t)col] |= 1u << int(t / ((long long)ktiles.nt1 * ktiles.nt2));
+          const size_t col = size_t(t) % cols, z = size_t(t) / cols;
+          cm[(z >> 5) * cols + col] |= 1u << (z & 31);
+          any[col] = 1;
         }
-      for (uint32_t v : cm) ncol += v != 0u;
-      p->kcol_fraction = double(ncol) / double(cm.size());
+      long long ncol = 0;
+      for (char v : any) ncol += v;
+      p->kcol_fraction = ktiles.nt0 <= 32 ? double(ncol) / double(cols) : 1.0;
       NRS_TRY(dev_alloc_n(p, &p->kcolmask, (long long)cm.size()));
       NRS_TRY(upload(p->kcolmask, cm, s));
+      std::vector<uint32_t> am((size_t)ktiles.nt2 * ((ktiles.nt1 + 31) / 32), 0u);
+      for (size_t c = 0; c < cols; ++c)
+        if (any[c]) {
+          const size_t y = c / ktiles.nt2;
+          am[(y >> 5) * ktiles.nt2 + c % ktiles.nt2] |= 1u << (y & 31);
+        }
+      NRS_TRY(dev_alloc_n(p, &p->kanymask, (long long)am.size()));
+      NRS_TRY(upload(p->kanymask, am, s));
     }
     for (int j = 0; j < p->P; ++j) {
       NRS_TRY(build_pointset(p, all[(size_t)j], &p->kpts[j], ktiles, &uni, /*interp=*/true,
@@ -783,6 +828,7 @@ nrsense_status create_impl(nrsense_plan_s* p, const nrsense_desc* desc, const in
     p->image_fft_ok = pruned_image_fft_supported(g) && !p->comp_spread;
     p->image_fft_pruned = p->image_fft_ok;
   }
+  NRS_TRY(create_mixed(p, s));
   if (p->C > 0) {
     const size_t cgb = size_t(g.ngrid) * p->C * p->phase_chunk * (p->grid_bf16 ? 4 : 8);
     NRS_TRY(dev_alloc(p, &p->b_xpad, cgb));
@@ -794,6 +840,11 @@ nrsense_status create_impl(nrsense_plan_s* p, const nrsense_desc* desc, const in
     // times both paths)
     p->fft_pruned_ok = pruned_fft_supported(g, p->C, p->grid_bf16) && init_pruned_fft() == cudaSuccess;
     p->fft_pruned = p->fft_pruned_ok;
+    // power-of-two grids: the mixed-radix kernels are the faster ones with 128
+    // points (64^3, 8 coils, 2 phases: 0.256 against 0.294 ms per E), the
+    // power-of-two ones with 256 (128^3, 4 phases: 3.16 against 3.45) and,
+    // barely, with 32 and 64
+    p->coil_mixed = p->mix[0].N > 0 && (!p->fft_pruned_ok || std::max(g.g0, std::max(g.g1, g.g2)) == 128);
     // tensor maps of the interpolation input (TMA-staged halos, W = 4)
     const long long slots = (long long)p->C * p->phase_chunk;
     // a test-only limit on the halo wait (0 makes every TMA-staged CTA time out)

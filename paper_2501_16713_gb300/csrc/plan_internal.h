@@ -47,6 +47,34 @@ struct PointSet {
 
 }  // namespace nrs
 
+namespace nrs {
+// One transform length of the mixed-radix passes (fft_mixed.cuh): L = r1 r2 r3,
+// s = r2 r3, ceil(2^32 / d) of the divisors d its index arithmetic needs.
+struct MixLen {
+  int L, r1, r2, r3, s;
+  unsigned m_s, m_13, m_12, m_r3, m_r1;
+  const float2* tw;  // exp(-2 pi i j / L), j < L (device)
+};
+// One axis: N = R S data values, G = 2N (R > 0), or any N and G with the radices
+// of both lengths (R = 0); exp(-2 pi i j / G) and exp(-2 pi i j / N) (device).
+struct MixAxis {
+  int N, G, R, S;
+  MixLen g, n;
+  const float2 *tw_g, *tw_n;
+};
+// One pass over one axis (fft_mixed_kernels.cuh: run_pass).
+struct MixPass {
+  const Geo* geo;
+  int pass, C, nph;
+  const uint32_t* colmask;  // z passes: plan's kcolmask, y passes: kanymask
+  const float* deapod;
+  const nrsense_c64* smaps;
+  const void* in;
+  void* out;
+  bool configure;  // only allow the pass' kernel its shared memory
+};
+}  // namespace nrs
+
 struct nrsense_cg_ws;  // CG workspace (solver.cu)
 struct nrsense_fista_ws;  // FISTA workspace (fista.cu)
 struct nrsense_motion_ws;  // density compensation / weighted adjoint workspace (motion.cu)
@@ -142,12 +170,24 @@ struct nrsense_plan_s {
   bool image_fft_ok = false;
   bool image_fft_pruned = false;
   bool upad_dirty = false;
+  // mixed-radix passes (fft_mixed.cu): coil_mixed: the own coil-grid transforms
+  // are these (else the power-of-two ones); image_mixed: so are those of T / T^H
+  nrs::MixAxis mix[3] = {};
+  bool coil_mixed = false;
+  bool image_mixed = false;
+  // own coil-grid transforms in use (where the power-of-two ones do not apply,
+  // the mixed-radix ones are always; the tuning choice is about the former)
+  bool own_fft() const { return fft_pruned || (coil_mixed && !fft_pruned_ok); }
+  bool own_image_fft() const { return image_fft_pruned || (image_mixed && !image_fft_ok); }
   bool pad_dirty = false;      // b_xpad / b_xmid hold the pruned transforms' intermediates
-  // k-space tiles written by the spread (the union over phases), as one
-  // 32-bit mask over axis-0 tiles per (axis-1, axis-2) tile column; null when
-  // axis 0 has more than 32 tiles.  Tiles outside it are zero in the spread
+  // k-space tiles written by the spread (the union over phases), as masks over
+  // axis-0 tiles per (axis-1, axis-2) tile column: word w (32 tiles each) of all
+  // columns, then word w + 1.  Tiles outside it are zero in the spread
   // target and never read by the interpolation.
   uint32_t* kcolmask = nullptr;
+  // per axis-2 tile, masks over axis-1 tiles of the columns that have such a tile
+  // (word w of all axis-2 tiles, then word w + 1)
+  uint32_t* kanymask = nullptr;
   double kcol_fraction = 1.0;  // tile columns with at least one such tile
   double kuni_fraction = 1.0;  // tiles of the union
 
@@ -305,13 +345,39 @@ int launch_pruned_image_adjoint(const Geo& g, const float* deapod, const nrsense
                                 void* t2, void* t1, nrsense_c64* xhat, cudaStream_t s);
 cudaError_t init_pruned_fft();
 int launch_pruned_forward(const Geo& g, int C, int nph, const uint32_t* colmask,
-                          const float* deapod,
+                          const uint32_t* anymask, const float* deapod,
                           const nrsense_c64* smaps, const nrsense_c64* m, void* t1, void* t2,
                           void* grid, cudaStream_t s);
 int launch_pruned_inverse(const Geo& g, int C, int nph, const uint32_t* colmask,
-                          const float* deapod,
+                          const uint32_t* anymask, const float* deapod,
                           const nrsense_c64* smaps, const void* grid, void* t2, void* t1,
                           nrsense_c64* w, cudaStream_t s);
+// mixed-radix transforms (fft_mixed.cu) of every axis that mix_axis accepts.
+// Coil grids as launch_pruned_*; image space: u = F_G^-1 Z (1/C) F_N x / N^3 and
+// its adjoint, with scratch t1 (N0 N1 G2 values, may be u: the pass that writes
+// u no longer reads t1) and t2 (N0 G1 G2 values).
+bool mix_axis(int N, int G, MixAxis* out);
+size_t mixed_max_smem(const MixAxis* ax);  // bound on the shared memory of the passes
+constexpr size_t kMixedMaxSmem = 224 * 1024;
+cudaError_t configure_mixed(const Geo& g, const MixAxis* ax);
+inline unsigned mix_magic(int d) { return unsigned(((1ull << 32) + unsigned(d) - 1) / unsigned(d)); }
+bool mixed_static_pass(const MixPass& a, const MixAxis& x, cudaStream_t s);  // false: no such radices
+void mixed_rt_coil_pass(const MixPass& a, const MixAxis& x, cudaStream_t s);
+void mixed_rt_image_pass(const MixPass& a, const MixAxis& x, cudaStream_t s);
+void mixed_gen_coil_pass(const MixPass& a, const MixAxis& x, cudaStream_t s);
+void mixed_gen_image_pass(const MixPass& a, const MixAxis& x, cudaStream_t s);
+int launch_mixed_forward(const Geo& g, const MixAxis* ax, int C, int nph, const uint32_t* colmask,
+                         const uint32_t* anymask, const float* deapod, const nrsense_c64* smaps, const nrsense_c64* m,
+                         void* t1, void* t2, void* grid, cudaStream_t s);
+int launch_mixed_inverse(const Geo& g, const MixAxis* ax, int C, int nph, const uint32_t* colmask,
+                         const uint32_t* anymask, const float* deapod, const nrsense_c64* smaps, const void* grid, void* t2,
+                         void* t1, nrsense_c64* w, cudaStream_t s);
+int launch_mixed_image_up(const Geo& g, const MixAxis* ax, const float* deapod,
+                          const nrsense_c64* x, void* t1, void* t2, nrsense_c64* u,
+                          cudaStream_t s);
+int launch_mixed_image_down(const Geo& g, const MixAxis* ax, const float* deapod,
+                            const nrsense_c64* u, void* t2, void* t1, nrsense_c64* x,
+                            cudaStream_t s);
 // rebuild the k-space spreading work items of every phase with at most
 // max_item list entries per item (plan.cu; the lists of split tiles are
 // re-dealt, the sorted points stay) and grow the split-tile scratch if needed
