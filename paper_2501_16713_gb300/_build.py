@@ -41,9 +41,10 @@ SOURCES = [
     "fft_mixed_gen_coil.cu",
     "fft_mixed_gen_image.cu",
     "spread_home.cu",
+    "spread_rows.cu",
 ]
 HEADERS = ["common.cuh", "plan_internal.h", "kb_host.h", "fft_mixed.cuh",
-           "fft_mixed_kernels.cuh"]
+           "fft_mixed_kernels.cuh", "mma_tf32.cuh"]
 
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 

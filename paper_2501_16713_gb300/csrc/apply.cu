@@ -254,7 +254,9 @@ nrsense_status warp_adjoint(nrsense_plan_s* p, const nrsense_c64* m, nrsense_c64
     STAGE(VECTOR, launch_sum_phases(g, p->P, m, x, s));
     return launched();
   }
-  if (p->spread_image_variant == kSpreadHome && p->home_ok) {
+  if (p->spread_rows()) {
+    STAGE(SPREAD_IMAGE, launch_spread_rows(g, p->W, p->kc, p->irows, m, p->b_ugrid, s));
+  } else if (p->spread_image_variant == kSpreadHome && p->home_ok) {
     STAGE(SPREAD_IMAGE, launch_spread_home(g, p->kc, p->ihome, m, p->b_ugrid, p->home_scratch, s));
   } else {
     const PhaseTable t = image_table(p);
@@ -513,7 +515,9 @@ nrsense_status nrsense_plan_autotune(nrsense_plan_t p, int32_t reps, nrsense_tun
     for (int k = 0; k < 3; ++k) {
       if (iv[k] == kSpreadHome && !p->home_ok) break;
       auto run = [&] {
-        if (iv[k] == kSpreadHome)
+        if (iv[k] == kSpreadHome && p->rows_sparse)
+          p->launches += launch_spread_rows(g, p->W, p->kc, p->irows, p->b_m, p->b_ugrid, s);
+        else if (iv[k] == kSpreadHome)
           p->launches += launch_spread_home(g, p->kc, p->ihome, p->b_m, p->b_ugrid,
                                             p->home_scratch, s);
         else

@@ -11,12 +11,14 @@ namespace nrs {
 
 // Coefficients of the per-tap kernel polynomials (see kb_host.cu):
 // weight of tap t for fractional offset f in [0, 1) is
-//   c(f + W/2 - 1 - t) ~= sum_k coef[t][k] * s^k,  s = 2f - 1.
+//   c(f + W/2 - 1 - t) ~= sum_k coef[k][t] * s^k,  s = 2f - 1.
+// The taps of one power are neighbours, so that two taps' coefficients load and
+// multiply as a pair.
 constexpr int kNumCoef = 10;
 constexpr int kMaxWidth = 6;
 
-struct KernelCoefs {
-  float c[kMaxWidth][kNumCoef];
+struct alignas(8) KernelCoefs {
+  float c[kNumCoef][kMaxWidth];
 };
 
 // Per-axis geometry passed by value to every kernel.
@@ -98,6 +100,16 @@ struct HomeSet {
   const int4* cover2;
 };
 
+// Image-space points (the displaced voxels of all phases) sorted by the 4^3
+// block of their first tap, row-major blocks, grids of a multiple of 4 points
+// per axis (spread_rows.cu).
+struct RowSet {
+  const float4* qs;       // sorted: (f0, f1, f2, packed first tap)
+  const int32_t* perm;    // sorted index -> value row
+  const int32_t* start;   // per block: first sorted index (nb0 nb1 nb2 + 1 entries)
+  int nb0, nb1, nb2;      // blocks per axis (G / 4)
+};
+
 // Phase slot of work item `i` of a launch (linear search; nphase is small).
 __device__ __forceinline__ int phase_of(const int* prefix, int nphase, int i) {
   int jj = 0;
@@ -113,15 +125,51 @@ struct ReduceItem {
   int32_t pad;
 };
 
-// Evaluate the W kernel weights of one axis for fractional offset f.
+// Evaluate the W kernel weights of the three axes for fractional offsets f0, f1,
+// f2, two taps per paired FMA (each part rounded as fmaf).  Home-tile spread of
+// four phases at 256^3: 0.605 -> 0.590 ms; the halo-list spreads, whose
+// accumulators fill the registers, are faster with one axis at a time
+// (register kernel at 128^3, 8 coils: 0.540 against 0.560 ms).
+template <int W>
+__device__ __forceinline__ void kernel_weights3(float f0, float f1, float f2, const KernelCoefs& kc,
+                                                float (&w0)[W], float (&w1)[W], float (&w2)[W]) {
+  static_assert(W % 2 == 0, "tap pairs");
+  const float f[3] = {f0, f1, f2};
+  float2 s[3], acc[3][W / 2];
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    const float v = fmaf(2.0f, f[a], -1.0f);
+    s[a] = make_float2(v, v);
+  }
+#pragma unroll
+  for (int k = kNumCoef - 1; k >= 0; --k)
+#pragma unroll
+    for (int t = 0; t < W / 2; ++t) {
+      const float2 c = *reinterpret_cast<const float2*>(&kc.c[k][2 * t]);
+#pragma unroll
+      for (int a = 0; a < 3; ++a)
+        acc[a][t] = k == kNumCoef - 1 ? c : __ffma2_rn(acc[a][t], s[a], c);
+    }
+#pragma unroll
+  for (int t = 0; t < W / 2; ++t) {
+    w0[2 * t] = acc[0][t].x;
+    w0[2 * t + 1] = acc[0][t].y;
+    w1[2 * t] = acc[1][t].x;
+    w1[2 * t + 1] = acc[1][t].y;
+    w2[2 * t] = acc[2][t].x;
+    w2[2 * t + 1] = acc[2][t].y;
+  }
+}
+
+// The W kernel weights of one axis.
 template <int W>
 __device__ __forceinline__ void kernel_weights(float f, const KernelCoefs& kc, float (&w)[W]) {
   const float s = fmaf(2.0f, f, -1.0f);
 #pragma unroll
   for (int t = 0; t < W; ++t) {
-    float acc = kc.c[t][kNumCoef - 1];
+    float acc = kc.c[kNumCoef - 1][t];
 #pragma unroll
-    for (int k = kNumCoef - 2; k >= 0; --k) acc = fmaf(acc, s, kc.c[t][k]);
+    for (int k = kNumCoef - 2; k >= 0; --k) acc = fmaf(acc, s, kc.c[k][t]);
     w[t] = acc;
   }
 }

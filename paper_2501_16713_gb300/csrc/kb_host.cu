@@ -104,13 +104,13 @@ double fit_kernel_polys(int width, double beta, KernelCoefs* out) {
       b[i] = kb_kernel(f + 0.5 * width - 1.0 - t, width, beta);
     }
     solve_dense(V, b, n);
-    for (int k = 0; k < n; ++k) out->c[t][k] = float(b[k]);
+    for (int k = 0; k < n; ++k) out->c[k][t] = float(b[k]);
     // error of the FP32 Horner evaluation (as on the GPU) against FP64 c
     for (int i = 0; i <= 4000; ++i) {
       const float f = float(i) / 4000.0f;
       const float s = std::fmaf(2.0f, f, -1.0f);
-      float acc = out->c[t][n - 1];
-      for (int k = n - 2; k >= 0; --k) acc = std::fmaf(acc, s, out->c[t][k]);
+      float acc = out->c[n - 1][t];
+      for (int k = n - 2; k >= 0; --k) acc = std::fmaf(acc, s, out->c[k][t]);
       const double ref = kb_kernel(double(f) + 0.5 * width - 1.0 - t, width, beta);
       worst = std::fmax(worst, std::fabs(double(acc) - ref) / peak);
     }

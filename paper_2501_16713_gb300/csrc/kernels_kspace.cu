@@ -105,7 +105,7 @@ __global__ void __launch_bounds__(256) interp_tile_kernel(
   const int tx = rem - ty * tp.nt2;
   const int o0 = tz * T, o1 = ty * T, o2 = tx * T;
   if (threadIdx.x < W * kNumCoef) s_coef[threadIdx.x / kNumCoef][threadIdx.x % kNumCoef] =
-      kc.c[threadIdx.x / kNumCoef][threadIdx.x % kNumCoef];
+      kc.c[threadIdx.x % kNumCoef][threadIdx.x / kNumCoef];
   // stage: lanes walk (coil, x) with the coil fastest, so shared writes are
   // contiguous and each global sector (4 consecutive x of one coil) is fully used
   for (int i = threadIdx.x; i < CC * H3; i += blockDim.x) {
@@ -284,7 +284,7 @@ __global__ void __launch_bounds__(256, CC == 2 ? 6 : CC == 4 ? 4 : 1) interp_tma
   const int tx = rem - ty * tp.nt2;
   const int o0 = tz * T, o1 = ty * T, o2 = tx * T;
   if (threadIdx.x < W * kNumCoef) s_coef[threadIdx.x / kNumCoef][threadIdx.x % kNumCoef] =
-      kc.c[threadIdx.x / kNumCoef][threadIdx.x % kNumCoef];
+      kc.c[threadIdx.x % kNumCoef][threadIdx.x / kNumCoef];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int grp = lane / LPS;          // sample slot in the warp
   const int gl = lane - grp * LPS;     // lane in the group

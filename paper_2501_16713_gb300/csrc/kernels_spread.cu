@@ -21,6 +21,7 @@
 // (FMA residual) and of every addition (TwoSum) is summed in a companion
 // array and added at write-out), which removes the growth of the
 // accumulation error with the number of points per grid value.
+#include "mma_tf32.cuh"
 #include "plan_internal.h"
 
 namespace nrs {
@@ -420,34 +421,8 @@ __global__ void __launch_bounds__(32 * WPC, WPC == 1 ? 24 : 3) spread_coils_reg_
 // hi.hi + hi.lo + lo.hi are accumulated, which keeps the error near FP32
 // rounding (the dropped lo.lo term is below 2^-22 relative).  The summation
 // order differs from the FMA kernels, so the result is not bitwise theirs.
-// Fragment layouts (PTX, m16n8k8 .tf32): g = lane / 4, q = lane % 4;
-// A: a0 (g, q), a1 (g + 8, q), a2 (g, q + 4), a3 (g + 8, q + 4);
-// B: b0 (k = q, n = g), b1 (k = q + 4, n = g);
-// C: c0, c1 (g, 2q, 2q + 1), c2, c3 (g + 8, 2q, 2q + 1).
-__device__ __forceinline__ uint32_t tf32_rna(float x) {
-  uint32_t r;
-  asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(r) : "f"(x));
-  return r;
-}
-
-// x = hi + lo: hi = x rounded to TF32; the remainder x - hi is exact in FP32
-// and goes to the tensor core as it is (no second rounding: one instruction
-// less per operand element), which uses its TF32 part, within 2^-10 of it,
-// i.e. within 2^-21 of x.
-__device__ __forceinline__ void split_tf32(float x, uint32_t& hi, uint32_t& lo) {
-  hi = tf32_rna(x);
-  lo = __float_as_uint(x - __uint_as_float(hi));
-}
-
-__device__ __forceinline__ void mma_tf32(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2,
-                                         uint32_t a3, uint32_t b0, uint32_t b1) {
-  asm volatile(
-      "mma.sync.aligned.m16n8k8.row.col.f32.tf32.tf32.f32 {%0, %1, %2, %3}, "
-      "{%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};\n"
-      : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-      : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
-}
-
+// Split, product and fragment layouts: mma_tf32.cuh.
+//
 // WPC warps per CTA, warp w serving plane (blockIdx.x * WPC + w) % 8 of item
 // (blockIdx.x * WPC + w) / 8 (WPC divides 8).
 template <typename GT, int WPC>
@@ -696,9 +671,7 @@ __global__ void __launch_bounds__(32 * WPC, 28 / WPC) spread_coils_cube_kernel(
         if (r2 < 0) r2 += g.g2;
         if (r2 >= T) r2 -= g.g2;
         float wz[W], wy[W], wx[W];
-        kernel_weights<W>(qq.x, kc, wz);
-        kernel_weights<W>(qq.y, kc, wy);
-        kernel_weights<W>(qq.z, kc, wx);
+        kernel_weights3<W>(qq.x, qq.y, qq.z, kc, wz, wy, wx);
         CubeStage& d = stg[lane];
         reinterpret_cast<float4*>(d.wz)[0] = make_float4(wz[0], wz[1], wz[2], wz[3]);
         reinterpret_cast<float4*>(d.wy)[0] = make_float4(wy[0], wy[1], wy[2], wy[3]);

@@ -491,6 +491,52 @@ nrsense_status build_home_set(nrsense_plan_s* p, const std::vector<HostPoint>& p
   return NRSENSE_OK;
 }
 
+// Image-space points sorted by the 4^3 block of their first tap (stable), with
+// the first sorted index of every block (spread_rows.cu).
+nrsense_status build_row_set(nrsense_plan_s* p, const std::vector<HostPoint>& pts, cudaStream_t s) {
+  const Geo& g = p->geo;
+  RowSet& rs = p->irows;
+  rs.nb0 = g.g0 / 4;
+  rs.nb1 = g.g1 / 4;
+  rs.nb2 = g.g2 / 4;
+  const size_t nblk = (size_t)rs.nb0 * rs.nb1 * rs.nb2, n = pts.size();
+  auto block = [&](const HostPoint& h) {
+    return ((size_t)(h.b[0] >> 2) * rs.nb1 + (h.b[1] >> 2)) * rs.nb2 + (h.b[2] >> 2);
+  };
+  std::vector<int32_t> start(nblk + 1, 0), at(nblk);
+  for (const HostPoint& h : pts) start[block(h) + 1]++;
+  for (size_t b = 0; b < nblk; ++b) start[b + 1] += start[b];
+  std::copy(start.begin(), start.end() - 1, at.begin());
+  std::vector<float4> qs(std::max<size_t>(n, 1));
+  std::vector<int32_t> perm(std::max<size_t>(n, 1));
+  for (const HostPoint& h : pts) {
+    const size_t k = size_t(at[block(h)]++);
+    const uint32_t packed = pack_base(h.b[0], h.b[1], h.b[2]);
+    float w;
+    std::memcpy(&w, &packed, sizeof(w));
+    qs[k] = make_float4(h.f[0], h.f[1], h.f[2], w);
+    perm[k] = h.row;
+  }
+  float4* dq = nullptr;
+  int32_t *dp = nullptr, *ds = nullptr;
+  NRS_TRY(dev_alloc_n(p, &dq, (long long)qs.size()));
+  NRS_TRY(dev_alloc_n(p, &dp, (long long)perm.size()));
+  NRS_TRY(dev_alloc_n(p, &ds, (long long)start.size()));
+  NRS_TRY(upload(dq, qs, s));
+  NRS_TRY(upload(dp, perm, s));
+  NRS_TRY(upload(ds, start, s));
+  rs.qs = dq;
+  rs.perm = dp;
+  rs.start = ds;
+  p->rows_ok = true;
+  // rows against home tiles, points per grid value: 1/8 (one phase at sigma 2)
+  // 0.695 against 1.08 ms at 384^3, 1/4 (two phases) 0.40 against 0.40 ms at
+  // 256^3, 1/2 0.76 against 0.59: the home tiles' fixed cost per tile
+  // (accumulators, merge, rims) against the rows' four visits per point
+  p->rows_sparse = p->W == 4 && 6 * (long long)n <= g.ngrid;
+  return NRSENSE_OK;
+}
+
 // scratch for split tiles: slots x coil chunks x tile x chunk coils (grown,
 // never shrunk)
 nrsense_status ensure_scratch(nrsense_plan_s* p) {
@@ -668,11 +714,12 @@ nrsense_status create_impl(nrsense_plan_s* p, const nrsense_desc* desc, const in
     }
     NRS_TRY(build_pointset(p, pts, &p->ipts, itiles, nullptr, /*interp=*/false,
                            kSpreadMaxItemImage, s));
+    if (!p->comp_spread && !p->grid_bf16 && g.g0 % 4 == 0 && g.g1 % 4 == 0 && g.g2 % 4 == 0)
+      NRS_TRY(build_row_set(p, pts, s));
     // home-tile spread (W = 4, plain FP32 accumulation); the default where built
     if (p->W == 4 && !p->comp_spread) {
       NRS_TRY(build_home_set(p, pts, s));
       p->spread_image_variant = kSpreadHome;
-      p->interp_home = true;
     }
   }
 

@@ -100,8 +100,14 @@ struct nrsense_plan_s {
   std::vector<nrs::PointSet> kpts;  // per phase
   nrs::PointSet ipts;               // displaced voxels of all phases
   nrs::HomeSet ihome{};             // the same, sorted by 8^3 home tile (home-tile spread)
+  nrs::RowSet irows{};              // the same, sorted by 4^3 block (row spread)
+  bool rows_ok = false;             // irows built (grids of a multiple of 4, plain FP32)
+  bool rows_sparse = false;         // rows_ok, W = 4 and few enough points for the row spread
   bool home_ok = false;             // ihome built (W = 4, not compensated)
-  bool interp_home = false;         // image-space interpolation over super-tiles (autotuned)
+  // image-space interpolation over super-tiles (autotuned; a thread per voxel
+  // until then: 0.324 against 0.414 ms at 192^3 with one phase, 0.300 against
+  // 0.309 at 128^3 with four, 0.0067 against 0.0148 at 32^3)
+  bool interp_home = false;
   nrsense_c64* home_scratch = nullptr;  // super-tile rims of the home-tile spread
   nrs::TilePlan ktiles{}, itiles{};  // k-space and image-space tiles
   int phase_chunk = 1;              // phases per launch
@@ -178,6 +184,12 @@ struct nrsense_plan_s {
   // own coil-grid transforms in use (where the power-of-two ones do not apply,
   // the mixed-radix ones are always; the tuning choice is about the former)
   bool own_fft() const { return fft_pruned || (coil_mixed && !fft_pruned_ok); }
+  // the image-space spread runs by block rows: always for W = 6 (the alternative
+  // is the generic halo-list kernel), for W = 4 as the kSpreadHome choice of
+  // sparse plans
+  bool spread_rows() const {
+    return rows_ok && (W != 4 || (rows_sparse && spread_image_variant == 5));
+  }
   bool own_image_fft() const { return image_fft_pruned || (image_mixed && !image_fft_ok); }
   bool pad_dirty = false;      // b_xpad / b_xmid hold the pruned transforms' intermediates
   // k-space tiles written by the spread (the union over phases), as masks over
@@ -327,6 +339,9 @@ int launch_spread_home(const Geo& g, const KernelCoefs& kc, const HomeSet& hs,
                        const nrsense_c64* vals, nrsense_c64* grid, nrsense_c64* scratch,
                        cudaStream_t s);
 long long home_scratch_elems(const HomeSet& hs);
+// row spread on the tensor cores (spread_rows.cu): all points of `rs` into grid
+int launch_spread_rows(const Geo& g, int W, const KernelCoefs& kc, const RowSet& rs,
+                       const nrsense_c64* vals, nrsense_c64* grid, cudaStream_t s);
 // image-space interpolation over the same super-tiles (spread_home.cu): m rows
 // perm of the home set's points, all phases
 int launch_interp_home(const Geo& g, const KernelCoefs& kc, const HomeSet& hs,

@@ -113,9 +113,7 @@ __global__ void __launch_bounds__(32 * kHWarps, 2)
         // the first tap lies in the home tile: offsets in [0, 8)
         const int r0 = b0 - h0, r1 = b1 - h1, r2 = b2 - h2;
         float wz[4], wy[4], wx[4];
-        kernel_weights<4>(q.x, kc, wz);
-        kernel_weights<4>(q.y, kc, wy);
-        kernel_weights<4>(q.z, kc, wx);
+        kernel_weights3<4>(q.x, q.y, q.z, kc, wz, wy, wx);
         float4* d = reinterpret_cast<float4*>(stg + lane);
         d[0] = make_float4(wz[0], wz[2], wz[1], wz[3]);
         d[1] = make_float4(wy[0], wy[1], wy[2], wy[3]);
@@ -333,9 +331,7 @@ __global__ void __launch_bounds__(256) interp_home_kernel(Geo g, KernelCoefs kc,
     int b0, b1, b2;
     unpack_base(__float_as_uint(q.w), b0, b1, b2);
     float w0[4], w1[4], w2[4];
-    kernel_weights<4>(q.x, kc, w0);
-    kernel_weights<4>(q.y, kc, w1);
-    kernel_weights<4>(q.z, kc, w2);
+    kernel_weights3<4>(q.x, q.y, q.z, kc, w0, w1, w2);
     const float2* base = reg + ((b0 - o0) * kHR + (b1 - o1)) * kHR + (b2 - o2);
     float2 aw = make_float2(0.f, 0.f);
 #pragma unroll
