@@ -626,6 +626,8 @@ nrsense_status nrsense_plan_autotune(nrsense_plan_t p, int32_t reps, nrsense_tun
                                    p->d_status, s);
     });
   const bool mma_ok = p->W == 4 && p->C > 4 && !p->comp_spread;
+  // up to 4 coils: the sub-block kernel of one to four coils takes that place
+  const bool few_ok = p->W == 4 && p->C > 1 && p->C <= 4 && !p->comp_spread && !p->grid_bf16;
   out->spread_mma_ms = -1.0;
   out->spread_mma_wpc = 0;
   out->spread_mma_cube = 0;
@@ -651,6 +653,13 @@ nrsense_status nrsense_plan_autotune(nrsense_plan_t p, int32_t reps, nrsense_tun
         }
       }
     }
+  }
+  if (few_ok) {
+    out->spread_mma_ms = time_ms([&] {
+      p->launches += launch_spread(g, p->W, p->kc, p->C, p->ktiles, ts, p->b_y, p->b_xspread, false,
+                                   false, spread_mma_variant(1, false), p->b_scratch, p->d_status, s);
+    });
+    out->spread_mma_wpc = 1;
   }
   const int chunks[2] = {8, 4};
   const bool saved_tma = p->interp_tma;
@@ -715,7 +724,7 @@ nrsense_status nrsense_plan_autotune(nrsense_plan_t p, int32_t reps, nrsense_tun
     for (int k = 1; k < 3; ++k)
       if (out->spread_ms[k] < out->spread_ms[bk]) bk = k;
     p->spread_variant = variants[bk];
-    if (mma_ok && out->spread_mma_ms >= 0.0 && out->spread_mma_ms < out->spread_ms[bk])
+    if ((mma_ok || few_ok) && out->spread_mma_ms >= 0.0 && out->spread_mma_ms < out->spread_ms[bk])
       p->spread_variant = spread_mma_variant(out->spread_mma_wpc, out->spread_mma_cube == 1);
   }
   // fastest interpolation: staging (per value / TMA) x coils per CTA (8 / 4; TMA also 2)

@@ -222,6 +222,52 @@ __global__ void __launch_bounds__(256) interp_tile_kernel(
   }
 }
 
+// K6 for one coil without tensor map (density compensation): four lanes per
+// sample gather their tap x straight from the grid; the samples of an item share
+// their lines in L1, and a heartbeat's few samples per tile do not pay for a
+// staged halo.  Sums in the order of interp_tile_kernel.
+template <int W>
+__global__ void __launch_bounds__(128) interp_one_kernel(Geo g, KernelCoefs kc, PhaseTable pt,
+                                                         const float2* __restrict__ grids,
+                                                         float2* __restrict__ y) {
+  constexpr int LPS = W == 4 ? 4 : 8;  // lanes per sample (W = 6: two idle)
+  const int jj = phase_of(pt.item0, pt.nphase, blockIdx.x);
+  const SpreadItem it = pt.items[jj][blockIdx.x - pt.item0[jj]];
+  const float2* __restrict__ grid = grids + (long long)jj * g.ngrid;
+  const int tx = threadIdx.x % LPS, sub = threadIdx.x / LPS;
+  const int txc = min(tx, W - 1);
+  for (int s0 = it.begin; s0 < it.end; s0 += 128 / LPS) {
+    const int s = min(s0 + sub, it.end - 1);
+    const float4 q = __ldg(pt.qs[jj] + s);
+    int b0, b1, b2;
+    unpack_base(__float_as_uint(q.w), b0, b1, b2);
+    float w0[W], w1[W], w2[W];
+    kernel_weights3<W>(q.x, q.y, q.z, kc, w0, w1, w2);
+    const float w2t = select_tap<W>(w2, txc);
+    const float2* col = grid + wrap_once(b2 + txc, g.g2);
+    float2 acc = make_float2(0.f, 0.f);
+#pragma unroll
+    for (int t0 = 0; t0 < W; ++t0) {
+      const float w02 = w0[t0] * w2t;
+      const long long row = (long long)wrap_once(b0 + t0, g.g0) * g.g1;
+#pragma unroll
+      for (int t1 = 0; t1 < W; ++t1) {
+        const float w = w02 * w1[t1];
+        const float2 v = __ldg(col + (row + wrap_once(b1 + t1, g.g1)) * g.g2);
+        acc.x = fmaf(w, v.x, acc.x);
+        acc.y = fmaf(w, v.y, acc.y);
+      }
+    }
+    if (tx >= W) acc = make_float2(0.f, 0.f);
+#pragma unroll
+    for (int off = 1; off < LPS; off <<= 1) {
+      acc.x += __shfl_xor_sync(0xffffffffu, acc.x, off);
+      acc.y += __shfl_xor_sync(0xffffffffu, acc.y, off);
+    }
+    if (tx == 0 && s0 + sub < it.end) y[pt.row0[jj] + __ldg(pt.perm[jj] + s)] = acc;
+  }
+}
+
 // K6 with the tile halo loaded by the tensor memory accelerator (W = 4).
 // One cp.async.bulk.tensor copy per CTA moves the (8+3)^3 halo of CC coil
 // grids (box x extent 12 for 16-byte rows) into shared memory as
@@ -636,6 +682,14 @@ int launch_interp_kspace(const Geo& g, int W, const KernelCoefs& kc, int C, cons
         interp_tma_kernel<4, float2><<<gd, 256, interp_tma_smem<4, float2>(), s>>>(
             *tmap, g, kc, C, tp, pt, gp, yp, status, lim);
     }
+    return 1;
+  }
+  if (C == 1 && !bf16) {
+    const auto* gp = static_cast<const float2*>(grids);
+    if (W == 4)
+      interp_one_kernel<4><<<nitems, 128, 0, s>>>(g, kc, pt, gp, yp);
+    else
+      interp_one_kernel<6><<<nitems, 128, 0, s>>>(g, kc, pt, gp, yp);
     return 1;
   }
   if (bf16)

@@ -344,11 +344,11 @@ nrsense_status build_pointset(nrsense_plan_s* p, std::vector<HostPoint>& pts, Po
     bk[nb - 1] = itm.end - itm.begin;
   }
   // class-ordered copy for the tensor-core spread over 4^3 sub-blocks (8^3
-  // tiles, W = 4): along each axis the first-tap offset r in [-3, 7] puts a
-  // footprint in the low half of the tile only (r <= 0), in both halves
-  // (1 <= r <= 3) or in the high half only (r >= 4); the entries of every item
+  // tiles): along each axis the first-tap offset r in [1 - W, 7] puts a
+  // footprint in the low half of the tile only (r <= 4 - W), in both halves
+  // (r <= 3) or in the high half only (r >= 4); the entries of every item
   // are ordered by class 9 c0 + 3 c1 + c2 (stable), with 28 offsets per item
-  const bool cube = W == 4 && tp.t0 == 8 && tp.t1 == 8 && tp.t2 == 8;
+  const bool cube = interp && tp.t0 == 8 && tp.t1 == 8 && tp.t2 == 8;
   std::vector<int2> clist2;
   std::vector<int32_t> cbins;
   if (cube) {
@@ -370,7 +370,7 @@ nrsense_status build_pointset(nrsense_plan_s* p, std::vector<HostPoint>& pts, Po
           int r = h.b[a] - o[a];
           if (r < 0) r += gsz[a];
           if (r >= 8) r -= gsz[a];
-          c = 3 * c + (r <= 0 ? 0 : r < 4 ? 1 : 2);
+          c = 3 * c + (r <= 4 - W ? 0 : r < 4 ? 1 : 2);
         }
         cls[i] = c;
         cb[c + 1]++;
@@ -900,6 +900,23 @@ nrsense_status create_impl(nrsense_plan_s* p, const nrsense_desc* desc, const in
                 make_grid_tensor_map(&p->tmap_xwork4, p->b_xwork, g, slots, p->grid_bf16, 4) &&
                 make_grid_tensor_map(&p->tmap_xwork8, p->b_xwork, g, slots, p->grid_bf16, 8) &&
                 make_grid_tensor_map(&p->tmap_xwork2, p->b_xwork, g, slots, p->grid_bf16, 2);
+    // launch choices until the plan is tuned.  Interpolation from TMA-staged halos
+    // of 4 coils (bitwise the per-value staging's results; 1.60 against 2.97 ms
+    // at 128^3, 8 coils, 4 phases; the tuned choice there).  FP32 spread by
+    // sub-blocks with FP32-accurate sums: on the tensor cores, eight points per
+    // rounded addition (5 to 8 coils and chunks of 8; 256^3, 16 coils, 3 M
+    // samples: 4.20 ms against 6.50 of the register kernel, the adjoint's error
+    // 2.6e-7 against 2.7e-7), or by FMAs (2 coils at 64^3, 100 k samples: 0.091 against
+    // 0.137 ms; with 3 and 4 coils the register kernel is the faster one on dense
+    // samples, 0.495 against 0.634 ms at 128^3, and the tuner times both).  The tuner's tensor-core
+    // candidate lets the tensor core accumulate, 4 % faster, with errors of a few
+    // 1e-6.  BF16 grids keep the register kernel and its exact summation order.
+    if (p->tma_ok) {
+      p->interp_tma = true;
+      p->interp_coils = p->C <= 2 ? 2 : 4;
+    }
+    if (p->W == 4 && !p->grid_bf16 && !p->comp_spread && (p->C <= 2 || p->C > 4))
+      p->spread_variant = kSpreadCubeExact;
     // empty tiles of the spread target are never written: zero them once
     if (cudaMemsetAsync(p->b_xspread, 0, cgb, s) != cudaSuccess) return NRSENSE_ERR_CUDA;
     NRS_TRY(dev_alloc_n(p, &p->b_y, std::max<long long>(p->Mtot * p->C, 1)));

@@ -317,7 +317,7 @@ int launch_crop_to_coils(const Geo& g, int C, const float* deapod, const void* x
 // shared-memory accumulation for the multi-coil W = 4 kernel (register
 // accumulation with a CTA per tile, or with a CTA per tile plane).
 constexpr int kSpreadRegister = 1, kSpreadShared = 2, kSpreadRegisterWarp = 3, kSpreadMMA = 4,
-              kSpreadHome = 5;
+              kSpreadHome = 5, kSpreadCubeExact = 6;
 // a spread variant value carries, in bits 8-15, the warps per CTA of the
 // tensor-core kernel (1, 2 or 4; 0 means 1) and, in bit 16, its geometry
 // (0: a warp per tile plane, 1: a warp per 4^3 sub-block)
