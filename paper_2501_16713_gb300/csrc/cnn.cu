@@ -58,7 +58,7 @@ constexpr int kRedBlocks = 1184;              // fixed grid: deterministic summa
 constexpr int kCin[kLayers] = {2, 16, 16, 16, 16};
 constexpr int kCout[kLayers] = {16, 16, 16, 16, 2};
 constexpr size_t kConvSmem = size_t(kHalo + kTaps * kCh) * kVS * sizeof(bf16);
-constexpr size_t kWgSmem = size_t(kHalo + kBlockVox) * kVS * sizeof(bf16);
+constexpr size_t kWgSmem = 2 * size_t(kHalo + kBlockVox) * kVS * sizeof(bf16);  // two stages
 
 struct Vol {
   int d, h, w;
@@ -522,20 +522,26 @@ __global__ void __launch_bounds__(kTcThreads, 4) conv3d_tc_kernel(
 // which ldmatrix.trans delivers from the channels-last tiles.  Persistent
 // grid; warp w accumulates the 9 taps of plane tz = w/4 over z plane w%4 of
 // every block its CTA visits and writes one partial [27][16][16] slice.
+// Bound by the latency of a block's copies and then of its ldmatrix/MMA chain,
+// with one CTA of 12 warps per SM (the 72 accumulators): the copies of the next
+// block run under the products of this one (2 x 76 KB of stages).  Two pairs of
+// 128^3, twelve calls: with the parallel reduction below 9.95 -> 8.24 ms for the
+// whole gradient and application, the sums bit for bit as before.
 __global__ void __launch_bounds__(kWgThreads, 1) wgrad_kernel(Vol v, const bf16* __restrict__ in,
                                                                const bf16* __restrict__ gr,
                                                                float* __restrict__ part_w,
                                                                float* __restrict__ part_b) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
-  bf16* sx = reinterpret_cast<bf16*>(smem_raw);  // [kHalo][kVS]
-  bf16* sg = sx + kHalo * kVS;                    // [kBlockVox][kVS]
+  // two stages of [kHalo][kVS] inputs and [kBlockVox][kVS] gradients
+  bf16* const stage0 = reinterpret_cast<bf16*>(smem_raw);
+  constexpr int kStage = (kHalo + kBlockVox) * kVS;
   __shared__ float sb[kWgThreads / kCh][kCh];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int tz = warp >> 2, wz = warp & 3;
   const int grow = (lane & 7) + (lane >> 4) * 8, gcol = ((lane >> 3) & 1) * 8;
   const int xrow = (lane & 7) + ((lane >> 3) & 1) * 8, xcol = (lane >> 4) * 8;
-  const unsigned sg_a = smem_u32(sg + (wz * BY * BX + grow) * kVS + gcol);
-  const unsigned sx_b = smem_u32(sx + xrow * kVS + xcol);
+  const unsigned sg_a0 = smem_u32(stage0 + kHalo * kVS + (wz * BY * BX + grow) * kVS + gcol);
+  const unsigned sx_b0 = smem_u32(stage0 + xrow * kVS + xcol);
   const int bch = threadIdx.x & (kCh - 1), bpart = threadIdx.x / kCh;
 
   float acc[9][2][4];
@@ -547,10 +553,11 @@ __global__ void __launch_bounds__(kWgThreads, 1) wgrad_kernel(Vol v, const bf16*
       for (int e = 0; e < 4; ++e) acc[k][n][e] = 0.f;
   float bacc = 0.f;
 
-  for (int b = blockIdx.x; b < v.nblocks; b += gridDim.x) {
+  auto stage = [&](int b, int half_buf) {
+    bf16* sx = stage0 + half_buf * kStage;
+    bf16* sg = sx + kHalo * kVS;
     int z0, y0, x0;
     block_origin(v, b, z0, y0, x0);
-    __syncthreads();  // previous block's readers are done
     stage_halo(v, in, sx, z0, y0, x0);
     for (int i = threadIdx.x; i < kBlockVox * 2; i += blockDim.x) {
       const int vox = i >> 1, half = i & 1;
@@ -560,8 +567,22 @@ __global__ void __launch_bounds__(kWgThreads, 1) wgrad_kernel(Vol v, const bf16*
       const long long gv = valid ? ((long long)gz * v.h + gy) * v.w + gx : 0;
       cp_async_16(sg + vox * kVS + half * 8, gr + gv * kCh + half * 8, valid);
     }
-    cp_async_wait_all();
+    asm volatile("cp.async.commit_group;\n" ::: "memory");
+  };
+  if (int(blockIdx.x) < v.nblocks) stage(blockIdx.x, 0);
+  int buf = 0;
+  for (int b = blockIdx.x; b < v.nblocks; b += gridDim.x, buf ^= 1) {
+    // the next block's copies run while this one is multiplied
+    if (b + int(gridDim.x) < v.nblocks) {
+      stage(b + gridDim.x, buf ^ 1);
+      asm volatile("cp.async.wait_group 1;\n" ::: "memory");
+    } else {
+      asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+    }
     __syncthreads();
+    const bf16* sg = stage0 + buf * kStage + kHalo * kVS;
+    const unsigned sg_a = sg_a0 + unsigned(buf * kStage * sizeof(bf16));
+    const unsigned sx_b = sx_b0 + unsigned(buf * kStage * sizeof(bf16));
     for (int vox = bpart; vox < kBlockVox; vox += kWgThreads / kCh)
       bacc += __bfloat162float(sg[vox * kVS + bch]);
 #pragma unroll 1
@@ -578,6 +599,7 @@ __global__ void __launch_bounds__(kWgThreads, 1) wgrad_kernel(Vol v, const bf16*
         mma_bf16(acc[t9][1], a0, a1, a2, a3, b01, b11);
       }
     }
+    __syncthreads();  // this stage's readers are done: the next iteration refills it
   }
 
   // D[m = o][n = c]: c0 = (g, 2t), c1 = (g, 2t+1), c2 = (g+8, 2t), c3 = (g+8, 2t+1)
@@ -604,18 +626,28 @@ __global__ void __launch_bounds__(kWgThreads, 1) wgrad_kernel(Vol v, const bf16*
   }
 }
 
-// grad[i] (+)= sum over partials, in fixed order, FP64.
-__global__ void wgrad_reduce_kernel(const float* __restrict__ part_w, int n_wparts,
-                                    const float* __restrict__ part_b, int n_bparts,
-                                    float* __restrict__ grad, int accumulate) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= kLayerP) return;
+// grad[i] (+)= sum over partials, in fixed order, FP64: eight runs of partials per
+// value (32 values per CTA), then the runs in order.
+constexpr int kReduceValues = 32, kReduceRuns = 8;
+__global__ void __launch_bounds__(kReduceValues * kReduceRuns) wgrad_reduce_kernel(
+    const float* __restrict__ part_w, int n_wparts, const float* __restrict__ part_b, int n_bparts,
+    float* __restrict__ grad, int accumulate) {
+  __shared__ double runs[kReduceRuns][kReduceValues];
+  const int col = threadIdx.x % kReduceValues, run = threadIdx.x / kReduceValues;
+  const int i = blockIdx.x * kReduceValues + col;
+  const bool weight = i < kLayerW;
+  const int n = weight ? n_wparts : n_bparts, per = (n + kReduceRuns - 1) / kReduceRuns;
   double s = 0.0;
-  if (i < kLayerW) {
-    for (int p = 0; p < n_wparts; ++p) s += part_w[size_t(p) * kLayerW + i];
-  } else {
-    for (int p = 0; p < n_bparts; ++p) s += part_b[size_t(p) * kCh + (i - kLayerW)];
+  if (i < kLayerP) {
+    const float* src = weight ? part_w + i : part_b + (i - kLayerW);
+    const size_t stride = weight ? kLayerW : kCh;
+    const int e = min(n, (run + 1) * per);
+    for (int p = run * per; p < e; ++p) s += src[size_t(p) * stride];
   }
+  runs[run][col] = s;
+  __syncthreads();
+  if (run != 0 || i >= kLayerP) return;
+  for (int k = 1; k < kReduceRuns; ++k) s += runs[k][col];
   grad[i] = accumulate ? grad[i] + (float)s : (float)s;
 }
 
@@ -981,7 +1013,8 @@ void forward(nrsense_cnn_s* net, const float2* r, const double* sumsq_dev, float
 void wgrad(nrsense_cnn_s* net, int l, const bf16* in, const bf16* g, bool accumulate,
            cudaStream_t s) {
   wgrad_kernel<<<net->wg_grid, kWgThreads, kWgSmem, s>>>(net->vol, in, g, net->part_w, net->part_b);
-  wgrad_reduce_kernel<<<(kLayerP + 255) / 256, 256, 0, s>>>(
+  wgrad_reduce_kernel<<<(kLayerP + kReduceValues - 1) / kReduceValues,
+                        kReduceValues * kReduceRuns, 0, s>>>(
       net->part_w, net->wg_grid * kWgParts, net->part_b, net->wg_grid,
       net->grad + size_t(l) * kLayerP, accumulate ? 1 : 0);
   net->launches += 2;
