@@ -24,6 +24,7 @@ INCLUDE = os.path.join(ROOT, "include")
 SOURCES = [
     "kb_host.cu",
     "plan.cu",
+    "plan_image.cu",
     "apply.cu",
     "kernels_image.cu",
     "kernels_kspace.cu",

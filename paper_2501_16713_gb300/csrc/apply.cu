@@ -461,7 +461,10 @@ nrsense_status nrsense_plan_set_tuning(nrsense_plan_t p, const nrsense_tuning* t
   if (m != 0 && m != 512 && m != 1024 && m != 2048) return NRSENSE_ERR_ARG;
   if (t->image_fft_pruned != 0 && t->image_fft_pruned != 1) return NRSENSE_ERR_ARG;
   if (t->image_fft_pruned == 1 && !p->image_fft_ok) return NRSENSE_ERR_ARG;
-  // the one step that can fail for want of memory comes first
+  // the steps that can fail for want of memory come first
+  NRS_TRY(ensure_image_sets(p, p->W == 4 && t->spread_image_warp != 2,
+                            t->interp_image_home == 1 || (t->spread_image_warp == 2 && !p->rows_sparse),
+                            nullptr));
   if (m != 0) NRS_TRY(retile_kspace(p, m, nullptr));
   p->spread_variant = t->spread_variant == NRSENSE_TUNE_SPREAD_REGISTER   ? kSpreadRegister
                       : t->spread_variant == NRSENSE_TUNE_SPREAD_SHARED ? kSpreadShared
@@ -507,6 +510,7 @@ nrsense_status nrsense_plan_autotune(nrsense_plan_t p, int32_t reps, nrsense_tun
   if (!p->identity_warp && p->ipts.tp.t0 == 16) {
     // image-space spread: CTA per tile or per plane pair, timed on the plan's
     // displaced voxels (values: the internal warped-image buffer)
+    NRS_TRY(ensure_image_sets(p, true, p->home_ok, s));
     cudaEvent_t a, b;
     if (cudaEventCreate(&a) != cudaSuccess || cudaEventCreate(&b) != cudaSuccess)
       return NRSENSE_ERR_CUDA;

@@ -13,7 +13,8 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
-#include <numeric>
+#include <system_error>
+#include <thread>
 #include <vector>
 
 #include "kb_host.h"
@@ -100,15 +101,14 @@ struct HostPoint {
 inline void decompose(double q, int G, int W, int* base, float* frac) {
   const double fl = std::floor(q);
   long long b = (long long)fl - (W / 2 - 1);
-  b %= G;
-  if (b < 0) b += G;
+  if (b < 0 || b >= G) {
+    b %= G;
+    if (b < 0) b += G;
+  }
   *base = int(b);
   *frac = float(q - fl);
 }
 
-inline int tile_of(int idx, int tile) { return idx / tile; }
-
-// Sort points into tiles, build halo lists and work items, upload.
 // Morton (Z-order) code of a tile, 10 bits per axis: work items in this
 // order keep neighbouring tiles (which share halo data) close in time.
 uint64_t morton3(const TilePlan& tp, long long tile) {
@@ -134,131 +134,141 @@ TilePlan make_tileplan(const Geo& g, int T) {
   return tp;
 }
 
+// Tiles (edge 1 << sh) along one axis of G points that the W taps from b touch: 1 or
+// 2, or up to 3 where they wrap past a ragged last tile.
+inline int touched_tiles(int b, int W, int G, int sh, int* out) {
+  if (b + W <= G) {  // no wrap: a footprint is no longer than a tile
+    out[0] = b >> sh;
+    out[1] = (b + W - 1) >> sh;
+    return out[1] == out[0] ? 1 : 2;
+  }
+  int n = 0;
+  for (int t = 0; t < W; ++t) {
+    int gi = b + t;
+    if (gi >= G) gi -= G;
+    const int ti = gi >> sh;
+    bool seen = false;
+    for (int k = 0; k < n; ++k) seen |= (out[k] == ti);
+    if (!seen) out[n++] = ti;
+  }
+  return n;
+}
+
 // Mark every tile touched by a footprint of the given points.
 void mark_touched_tiles(const nrsense_plan_s* p, const TilePlan& tp,
                         const std::vector<HostPoint>& pts, std::vector<char>& mask) {
   const Geo& g = p->geo;
-  const int gsz[3] = {g.g0, g.g1, g.g2};
-  const int tsz[3] = {tp.t0, tp.t1, tp.t2};
+  const int sh = tp.t0 == 16 ? 4 : 3;
   for (const HostPoint& h : pts) {
-    int tl[3][2], nt[3];
-    for (int a = 0; a < 3; ++a) {
-      nt[a] = 0;
-      for (int t = 0; t < p->W; ++t) {
-        int gi = h.b[a] + t;
-        if (gi >= gsz[a]) gi -= gsz[a];
-        const int ti = gi / tsz[a];
-        if (nt[a] == 0 || tl[a][nt[a] - 1] != ti) {
-          if (nt[a] < 2) tl[a][nt[a]++] = ti;
-        }
-      }
-    }
-    for (int a = 0; a < nt[0]; ++a)
-      for (int b = 0; b < nt[1]; ++b)
-        for (int c = 0; c < nt[2]; ++c)
-          mask[((long long)tl[0][a] * tp.nt1 + tl[1][b]) * tp.nt2 + tl[2][c]] = 1;
+    int t0[8], t1[8], t2[8];
+    const int n0 = touched_tiles(h.b[0], p->W, g.g0, sh, t0);
+    const int n1 = touched_tiles(h.b[1], p->W, g.g1, sh, t1);
+    const int n2 = touched_tiles(h.b[2], p->W, g.g2, sh, t2);
+    for (int a = 0; a < n0; ++a)
+      for (int b = 0; b < n1; ++b)
+        for (int c = 0; c < n2; ++c) mask[((long long)t0[a] * tp.nt1 + t1[b]) * tp.nt2 + t2[c]] = 1;
   }
 }
 
-// write_mask: tiles that must be written even without points of this set
-// (NULL = every tile).
+// The host side of a point set: what upload_pointset copies to the device.
+struct HostSet {
+  TilePlan tp{};
+  long long npts = 0, list_len = 0;
+  int occupied = 0, slots = 0;
+  bool cube = false;
+  std::vector<float4> qs;
+  std::vector<int32_t> perm, bins, cbins;
+  std::vector<int2> list, clist;
+  std::vector<SpreadItem> items, iitems;
+  std::vector<ReduceItem> reds;
+};
+
+// Sort points into tiles, build halo lists and work items (host only: the phases
+// of a plan run in threads of their own).
 // tp: tiles of this set; write_mask: tiles that must be written even without
 // points (NULL = every tile); interp: also build interpolation work items.
-nrsense_status build_pointset(nrsense_plan_s* p, std::vector<HostPoint>& pts, PointSet* ps,
-                              const TilePlan& tp, const std::vector<char>* write_mask,
-                              bool interp, int max_item, cudaStream_t s) {
-  const Geo& g = p->geo;
-  ps->tp = tp;
-  const int W = p->W;
+nrsense_status compute_pointset(const Geo& g, int W, const std::vector<HostPoint>& pts,
+                                const TilePlan& tp, const std::vector<char>* write_mask,
+                                bool interp, int max_item, HostSet* hs) {
+  hs->tp = tp;
   const long long npts = (long long)pts.size();
-  ps->npts = npts;
+  hs->npts = npts;
   if (npts >= (1ll << 31)) return NRSENSE_ERR_ARG;
+  const int gsz[3] = {g.g0, g.g1, g.g2};
+  const int sh = tp.t0 == 16 ? 4 : 3, tmask = (1 << sh) - 1;  // tiles of 8 or 16 points per axis
 
-  // primary key: tile of the first tap; secondary: cell inside the tile
-  std::vector<int64_t> key(npts);
-  for (long long i = 0; i < npts; ++i) {
-    const HostPoint& h = pts[i];
-    const long long t = ((long long)tile_of(h.b[0], tp.t0) * tp.nt1 + tile_of(h.b[1], tp.t1)) *
-                            tp.nt2 + tile_of(h.b[2], tp.t2);
-    const int cell = ((h.b[0] % tp.t0) * tp.t1 + (h.b[1] % tp.t1)) * tp.t2 + (h.b[2] % tp.t2);
-    key[i] = t * 4096 + cell;  // cell < T^3 <= 4096
-  }
-  std::vector<int32_t> order(npts);
-  std::iota(order.begin(), order.end(), 0);
-  std::stable_sort(order.begin(), order.end(),
-                   [&](int32_t a, int32_t b) { return key[a] < key[b]; });
-  // interpolation items: sorted ranges of points sharing a first-tap tile
-  std::vector<SpreadItem> iitems;
-  if (interp) {
-    long long b = 0;
-    while (b < npts) {
-      const long long t = key[order[b]] / 4096;
-      long long e = b;
-      while (e < npts && key[order[e]] / 4096 == t) ++e;
-      for (long long cb = b; cb < e; cb += kInterpMaxItem)
-        iitems.push_back({int32_t(t), int32_t(cb), int32_t(std::min(e, cb + kInterpMaxItem)), -1});
-      b = e;
+  // order: tile of the first tap, cell inside the tile, input order (counting
+  // sort by tile, then each tile's (cell, index) keys)
+  std::vector<int64_t> first(tp.ntiles + 1, 0);
+  auto tile_id = [&](const HostPoint& h) {
+    return ((long long)(h.b[0] >> sh) * tp.nt1 + (h.b[1] >> sh)) * tp.nt2 + (h.b[2] >> sh);
+  };
+  for (const HostPoint& h : pts) first[tile_id(h) + 1]++;
+  for (long long t = 0; t < tp.ntiles; ++t) first[t + 1] += first[t];
+  std::vector<uint64_t> ko((size_t)npts);
+  {
+    std::vector<int64_t> at(first.begin(), first.end() - 1);
+    for (long long i = 0; i < npts; ++i) {
+      const HostPoint& h = pts[(size_t)i];
+      const uint64_t cell =
+          ((uint64_t(h.b[0] & tmask) << sh | uint64_t(h.b[1] & tmask)) << sh) | uint64_t(h.b[2] & tmask);
+      ko[(size_t)at[tile_id(h)]++] = cell << 32 | uint64_t(i);
     }
+  }
+  for (long long t = 0; t < tp.ntiles; ++t)
+    if (first[t + 1] - first[t] > 1) std::sort(ko.begin() + first[t], ko.begin() + first[t + 1]);
+  // interpolation items: sorted ranges of points sharing a first-tap tile
+  std::vector<SpreadItem>& iitems = hs->iitems;
+  if (interp) {
+    for (long long t = 0; t < tp.ntiles; ++t)
+      for (long long cb = first[t]; cb < first[t + 1]; cb += kInterpMaxItem)
+        iitems.push_back({int32_t(t), int32_t(cb),
+                          int32_t(std::min<long long>(first[t + 1], cb + kInterpMaxItem)), -1});
     std::stable_sort(iitems.begin(), iitems.end(), [&](const SpreadItem& a, const SpreadItem& b) {
       return morton3(tp, a.tile) < morton3(tp, b.tile);
     });
   }
-  key.clear();
-  key.shrink_to_fit();
 
-  std::vector<float4> qs(npts);
-  std::vector<int32_t> perm(npts);
+  std::vector<float4>& qs = hs->qs;
+  std::vector<int32_t>& perm = hs->perm;
+  qs.resize((size_t)npts);
+  perm.resize((size_t)npts);
+  std::vector<uint32_t> base((size_t)npts);  // packed first taps in sorted order
   for (long long s_i = 0; s_i < npts; ++s_i) {
-    const HostPoint& h = pts[order[s_i]];
+    const HostPoint& h = pts[(size_t)(ko[(size_t)s_i] & 0xffffffffu)];
     const uint32_t packed = pack_base(h.b[0], h.b[1], h.b[2]);
     float w;
     std::memcpy(&w, &packed, sizeof(w));
-    qs[s_i] = make_float4(h.f[0], h.f[1], h.f[2], w);
-    perm[s_i] = h.row;
+    qs[(size_t)s_i] = make_float4(h.f[0], h.f[1], h.f[2], w);
+    perm[(size_t)s_i] = h.row;
+    base[(size_t)s_i] = packed;
   }
+  std::vector<uint64_t>().swap(ko);
+  auto axis0 = [&](int32_t si) { return int(base[(size_t)si] >> 20); };
 
   // halo lists: every tile touched by a point's W^3 footprint
-  const int gsz[3] = {g.g0, g.g1, g.g2};
-  const int tsz[3] = {tp.t0, tp.t1, tp.t2};
-  const int ntz[3] = {tp.nt0, tp.nt1, tp.nt2};
-  auto touched = [&](const HostPoint& h, int a, int* out) {
-    int n = 0;
-    for (int t = 0; t < W; ++t) {
-      int gi = h.b[a] + t;
-      if (gi >= gsz[a]) gi -= gsz[a];
-      const int ti = gi / tsz[a];
-      bool seen = false;
-      for (int k = 0; k < n; ++k) seen |= (out[k] == ti);
-      if (!seen) out[n++] = ti;
-    }
-    (void)ntz;
-    return n;
-  };
-  std::vector<int64_t> counts(tp.ntiles + 1, 0);
-  for (long long s_i = 0; s_i < npts; ++s_i) {
-    const HostPoint& h = pts[order[s_i]];
-    int t0[8], t1[8], t2[8];
-    const int n0 = touched(h, 0, t0), n1 = touched(h, 1, t1), n2 = touched(h, 2, t2);
+  auto each_tile = [&](uint32_t packed, auto&& f) {
+    int b0, b1, b2, t0[8], t1[8], t2[8];
+    unpack_base(packed, b0, b1, b2);
+    const int n0 = touched_tiles(b0, W, gsz[0], sh, t0), n1 = touched_tiles(b1, W, gsz[1], sh, t1),
+              n2 = touched_tiles(b2, W, gsz[2], sh, t2);
     for (int a = 0; a < n0; ++a)
       for (int b = 0; b < n1; ++b)
-        for (int c = 0; c < n2; ++c)
-          counts[((long long)t0[a] * tp.nt1 + t1[b]) * tp.nt2 + t2[c] + 1]++;
-  }
+        for (int c = 0; c < n2; ++c) f(((long long)t0[a] * tp.nt1 + t1[b]) * tp.nt2 + t2[c]);
+  };
+  std::vector<int64_t> counts(tp.ntiles + 1, 0);
+  for (long long s_i = 0; s_i < npts; ++s_i)
+    each_tile(base[(size_t)s_i], [&](long long t) { counts[t + 1]++; });
   for (long long t = 0; t < tp.ntiles; ++t) counts[t + 1] += counts[t];
   const long long list_len = counts[tp.ntiles];
   if (list_len >= (1ll << 31)) return NRSENSE_ERR_ARG;
   std::vector<int32_t> list(list_len);  // sorted indices; paired with rows below
-  std::vector<int64_t> fill(counts.begin(), counts.end() - 1);
-  for (long long s_i = 0; s_i < npts; ++s_i) {
-    const HostPoint& h = pts[order[s_i]];
-    int t0[8], t1[8], t2[8];
-    const int n0 = touched(h, 0, t0), n1 = touched(h, 1, t1), n2 = touched(h, 2, t2);
-    for (int a = 0; a < n0; ++a)
-      for (int b = 0; b < n1; ++b)
-        for (int c = 0; c < n2; ++c)
-          list[fill[((long long)t0[a] * tp.nt1 + t1[b]) * tp.nt2 + t2[c]]++] = int32_t(s_i);
+  {
+    std::vector<int64_t> fill(counts.begin(), counts.end() - 1);
+    for (long long s_i = 0; s_i < npts; ++s_i)
+      each_tile(base[(size_t)s_i], [&](long long t) { list[fill[t]++] = int32_t(s_i); });
   }
-  ps->list_len = list_len;
+  hs->list_len = list_len;
   // within each tile, order the points by the plane offset of their first tap
   // (axis 0) relative to the tile origin, so the spreading warp that owns a
   // plane finds its points in one contiguous range (stable: ties keep order)
@@ -271,7 +281,7 @@ nrsense_status build_pointset(nrsense_plan_s* p, std::vector<HostPoint>& pts, Po
       if (e - b < 2) continue;
       const int o0 = int(t / ((long long)tp.nt1 * tp.nt2)) * tp.t0;
       auto key = [&](int32_t si) {
-        int r = pts[order[si]].b[0] - o0;
+        int r = axis0(si) - o0;
         if (r < 0) r += g.g0;
         if (r >= tp.t0) r -= g.g0;
         return r + W - 1;
@@ -286,8 +296,8 @@ nrsense_status build_pointset(nrsense_plan_s* p, std::vector<HostPoint>& pts, Po
 
   // work items: occupied tiles, plus empty tiles in write_mask (they write
   // zeros); heavy tiles split
-  std::vector<SpreadItem> items;
-  std::vector<ReduceItem> reds;
+  std::vector<SpreadItem>& items = hs->items;
+  std::vector<ReduceItem>& reds = hs->reds;
   int slots = 0, occupied = 0;
   for (long long t = 0; t < tp.ntiles; ++t) {
     const long long b = counts[t], e = counts[t + 1];
@@ -316,15 +326,13 @@ nrsense_status build_pointset(nrsense_plan_s* p, std::vector<HostPoint>& pts, Po
   std::stable_sort(items.begin(), items.end(), [&](const SpreadItem& a, const SpreadItem& b) {
     return morton3(tp, a.tile) < morton3(tp, b.tile);
   });
-  ps->n_items = int(items.size());
-  ps->n_reduces = int(reds.size());
-  ps->n_slots = slots;
-  ps->n_occupied = occupied;
-  ps->n_iitems = int(iitems.size());
+  hs->slots = slots;
+  hs->occupied = occupied;
   // per item: first entry of each first-tap plane offset bin (list sorted by
   // r0 within every tile, so within every item)
   const int nb = W + tp.t0 + 1;
-  std::vector<int32_t> bins((size_t)items.size() * nb);
+  std::vector<int32_t>& bins = hs->bins;
+  bins.resize(items.size() * nb);
   for (size_t k = 0; k < items.size(); ++k) {
     const SpreadItem& itm = items[k];
     const int o0 = int(itm.tile / ((long long)tp.nt1 * tp.nt2)) * tp.t0;
@@ -333,7 +341,7 @@ nrsense_status build_pointset(nrsense_plan_s* p, std::vector<HostPoint>& pts, Po
     for (int bb = 0; bb < nb - 1; ++bb) {
       // advance past entries with r0 + W - 1 < bb
       while (e < itm.end) {
-        int r = pts[order[list[e]]].b[0] - o0;
+        int r = axis0(list[e]) - o0;
         if (r < 0) r += g.g0;
         if (r >= tp.t0) r -= g.g0;
         if (r + W - 1 >= bb) break;
@@ -349,8 +357,9 @@ nrsense_status build_pointset(nrsense_plan_s* p, std::vector<HostPoint>& pts, Po
   // (r <= 3) or in the high half only (r >= 4); the entries of every item
   // are ordered by class 9 c0 + 3 c1 + c2 (stable), with 28 offsets per item
   const bool cube = interp && tp.t0 == 8 && tp.t1 == 8 && tp.t2 == 8;
-  std::vector<int2> clist2;
-  std::vector<int32_t> cbins;
+  std::vector<int2>& clist2 = hs->clist;
+  std::vector<int32_t>& cbins = hs->cbins;
+  hs->cube = cube;
   if (cube) {
     clist2.resize(list_len);
     cbins.assign(items.size() * kCubeBins, 0);
@@ -364,10 +373,10 @@ nrsense_status build_pointset(nrsense_plan_s* p, std::vector<HostPoint>& pts, Po
       cls.resize(n);
       int32_t* cb = cbins.data() + k * kCubeBins;
       for (int i = 0; i < n; ++i) {
-        const HostPoint& h = pts[order[list[itm.begin + i]]];
-        int c = 0;
+        int hb[3], c = 0;
+        unpack_base(base[(size_t)list[itm.begin + i]], hb[0], hb[1], hb[2]);
         for (int a = 0; a < 3; ++a) {
-          int r = h.b[a] - o[a];
+          int r = hb[a] - o[a];
           if (r < 0) r += gsz[a];
           if (r >= 8) r -= gsz[a];
           c = 3 * c + (r <= 4 - W ? 0 : r < 4 ? 1 : 2);
@@ -383,39 +392,166 @@ nrsense_status build_pointset(nrsense_plan_s* p, std::vector<HostPoint>& pts, Po
       }
     }
   }
-  std::vector<int2> list2(list_len);
-  for (long long i = 0; i < list_len; ++i) list2[i] = make_int2(list[i], perm[list[i]]);
-  std::vector<int32_t>().swap(list);
+  hs->list.resize(list_len);
+  for (long long i = 0; i < list_len; ++i) hs->list[i] = make_int2(list[i], perm[list[i]]);
+  return NRSENSE_OK;
+}
 
-  NRS_TRY(dev_alloc_n(p, &ps->qs, std::max<long long>(npts, 1)));
-  NRS_TRY(dev_alloc_n(p, &ps->perm, std::max<long long>(npts, 1)));
-  NRS_TRY(dev_alloc_n(p, &ps->list, std::max<long long>(list_len, 1)));
-  NRS_TRY(dev_alloc_n(p, &ps->items, std::max<long long>((long long)items.size(), 1)));
-  NRS_TRY(dev_alloc_n(p, &ps->bins, std::max<long long>((long long)bins.size(), 1)));
-  NRS_TRY(dev_alloc_n(p, &ps->reduces, std::max<long long>((long long)reds.size(), 1)));
-  NRS_TRY(dev_alloc_n(p, &ps->iitems, std::max<long long>((long long)iitems.size(), 1)));
-  NRS_TRY(upload(ps->qs, qs, s));
-  NRS_TRY(upload(ps->perm, perm, s));
-  NRS_TRY(upload(ps->list, list2, s));
-  NRS_TRY(upload(ps->items, items, s));
-  NRS_TRY(upload(ps->bins, bins, s));
-  NRS_TRY(upload(ps->reduces, reds, s));
-  NRS_TRY(upload(ps->iitems, iitems, s));
-  if (cube) {
-    NRS_TRY(dev_alloc_n(p, &ps->clist, std::max<long long>(list_len, 1)));
-    NRS_TRY(dev_alloc_n(p, &ps->cbins, std::max<long long>((long long)cbins.size(), 1)));
-    NRS_TRY(upload(ps->clist, clist2, s));
-    NRS_TRY(upload(ps->cbins, cbins, s));
+nrsense_status upload_pointset(nrsense_plan_s* p, const HostSet& hs, PointSet* ps, cudaStream_t s) {
+  ps->tp = hs.tp;
+  ps->npts = hs.npts;
+  ps->list_len = hs.list_len;
+  ps->n_items = int(hs.items.size());
+  ps->n_reduces = int(hs.reds.size());
+  ps->n_slots = hs.slots;
+  ps->n_occupied = hs.occupied;
+  ps->n_iitems = int(hs.iitems.size());
+  auto put = [&](auto** dst, const auto& src) -> nrsense_status {
+    NRS_TRY(dev_alloc_n(p, dst, std::max<long long>((long long)src.size(), 1)));
+    return upload(*dst, src, s);
+  };
+  NRS_TRY(put(&ps->qs, hs.qs));
+  NRS_TRY(put(&ps->perm, hs.perm));
+  NRS_TRY(put(&ps->list, hs.list));
+  NRS_TRY(put(&ps->items, hs.items));
+  NRS_TRY(put(&ps->bins, hs.bins));
+  NRS_TRY(put(&ps->reduces, hs.reds));
+  NRS_TRY(put(&ps->iitems, hs.iitems));
+  if (hs.cube) {
+    NRS_TRY(put(&ps->clist, hs.clist));
+    NRS_TRY(put(&ps->cbins, hs.cbins));
   }
   return NRSENSE_OK;
+}
+
+nrsense_status build_pointset(nrsense_plan_s* p, const std::vector<HostPoint>& pts, PointSet* ps,
+                              const TilePlan& tp, const std::vector<char>* write_mask, bool interp,
+                              int max_item, cudaStream_t s) {
+  HostSet hs;
+  NRS_TRY(compute_pointset(p->geo, p->W, pts, tp, write_mask, interp, max_item, &hs));
+  return upload_pointset(p, hs, ps, s);
+}
+
+// f(j) for j < n in threads (at most one per core); the first failure's status.
+template <class F>
+nrsense_status for_phases(int n, F&& f) {
+  const int nt = std::min<int>(n, std::max(1u, std::thread::hardware_concurrency()));
+  std::vector<nrsense_status> st((size_t)n, NRSENSE_OK);
+  auto work = [&](int k) {
+    for (int j = k; j < n; j += nt) {
+      try {
+        st[(size_t)j] = f(j);
+      } catch (const std::bad_alloc&) {
+        st[(size_t)j] = NRSENSE_ERR_OOM;
+      }
+    }
+  };
+  std::vector<std::thread> pool;
+  int started = 1;
+  try {
+    for (; started < nt; ++started) pool.emplace_back(work, started);
+  } catch (const std::system_error&) {
+    // no more threads: this one takes the rest
+  }
+  work(0);
+  for (std::thread& t : pool) t.join();
+  for (int k = started; k < nt; ++k) work(k);
+  for (nrsense_status v : st)
+    if (v != NRSENSE_OK) return v;
+  return NRSENSE_OK;
+}
+
+// Displaced voxel positions from the plan's displacements, on the host.
+nrsense_status host_image_points(nrsense_plan_s* p, std::vector<HostPoint>& pts, cudaStream_t s) {
+  const Geo& g = p->geo;
+  const long long nd = (long long)p->P * 3 * g.nvox;
+  const double sigma = double(g.g0) / double(g.n0);
+  std::vector<float> hd((size_t)nd);
+  if (cudaMemcpyAsync(hd.data(), p->disp, size_t(nd) * sizeof(float), cudaMemcpyDeviceToHost, s) !=
+          cudaSuccess ||
+      cudaStreamSynchronize(s) != cudaSuccess)
+    return NRSENSE_ERR_CUDA;
+  for (long long i = 0; i < nd; ++i)
+    if (!std::isfinite(hd[i]) || std::fabs(hd[i]) > 1e6f) return NRSENSE_ERR_ARG;
+  pts.resize((size_t)(p->P * g.nvox));
+  const int gs[3] = {g.g0, g.g1, g.g2};
+  for (int j = 0; j < p->P; ++j) {
+    const float* dj = hd.data() + (long long)j * 3 * g.nvox;
+    for (long long v = 0; v < g.nvox; ++v) {
+      const int i2 = int(v % g.n2);
+      const int i1 = int((v / g.n2) % g.n1);
+      const int i0 = int(v / ((long long)g.n1 * g.n2));
+      const int ii[3] = {i0, i1, i2};
+      HostPoint& h = pts[(size_t)(j * g.nvox + v)];
+      for (int a = 0; a < 3; ++a) {
+        // q = sigma * (n + d) = sigma*n + sigma*d in FP64 (sigma*n exact)
+        const double q = sigma * double(ii[a]) + sigma * double(dj[a * g.nvox + v]);
+        decompose(q, gs[a], p->W, &h.b[a], &h.f[a]);
+      }
+      h.row = int32_t(j * g.nvox + v);
+    }
+  }
+  return NRSENSE_OK;
+}
+
+// The displaced voxels grouped by the block of edge 1 << shift of their first tap
+// (cells: by cell within it), stable: on the device (plan_image.cu), or on the
+// host where a group is too crowded for that.
+nrsense_status sorted_image_points(nrsense_plan_s* p, int shift, bool cells, const float4** qs,
+                                   const int32_t** perm, const int32_t** start, cudaStream_t s) {
+  const Geo& g = p->geo;
+  const int e = 1 << shift, m = e - 1;
+  const int nb1 = (g.g1 + m) / e, nb2 = (g.g2 + m) / e;
+  const size_t groups = (size_t)((g.g0 + m) / e) * nb1 * nb2;
+  const long long n = (long long)p->P * g.nvox;
+  float4* dq = nullptr;
+  int32_t *dp = nullptr, *ds = nullptr;
+  NRS_TRY(dev_alloc_n(p, &dq, n));
+  NRS_TRY(dev_alloc_n(p, &dp, n));
+  NRS_TRY(dev_alloc_n(p, &ds, (long long)groups + 1));
+  *qs = dq;
+  *perm = dp;
+  *start = ds;
+  if (fault_requested("upload")) return NRSENSE_ERR_CUDA;
+  bool bad = false, done = false;
+  NRS_TRY(sort_image_points(g, p->W, double(g.g0) / double(g.n0), n, p->disp, shift, cells, dq, dp, ds,
+                            &bad, &done, s));
+  if (bad) return NRSENSE_ERR_ARG;
+  if (done) return NRSENSE_OK;
+  std::vector<HostPoint> pts;
+  NRS_TRY(host_image_points(p, pts, s));
+  std::vector<std::pair<uint64_t, int32_t>> ko((size_t)n);  // (group, cell), index
+  std::vector<int32_t> st(groups + 1, 0);
+  for (long long i = 0; i < n; ++i) {
+    const HostPoint& h = pts[(size_t)i];
+    const uint64_t k = ((uint64_t)(h.b[0] >> shift) * nb1 + (h.b[1] >> shift)) * nb2 + (h.b[2] >> shift);
+    const uint64_t cell = cells ? (((h.b[0] & m) * e) + (h.b[1] & m)) * e + (h.b[2] & m) : 0;
+    ko[(size_t)i] = {k << 32 | cell, int32_t(i)};
+    st[(size_t)k + 1]++;
+  }
+  std::sort(ko.begin(), ko.end());
+  for (size_t k = 0; k < groups; ++k) st[k + 1] += st[k];
+  std::vector<float4> hq((size_t)n);
+  std::vector<int32_t> hp((size_t)n);
+  for (long long k = 0; k < n; ++k) {
+    const HostPoint& h = pts[(size_t)ko[(size_t)k].second];
+    const uint32_t packed = pack_base(h.b[0], h.b[1], h.b[2]);
+    float w;
+    std::memcpy(&w, &packed, sizeof(w));
+    hq[(size_t)k] = make_float4(h.f[0], h.f[1], h.f[2], w);
+    hp[(size_t)k] = h.row;
+  }
+  NRS_TRY(upload(dq, hq, s));
+  NRS_TRY(upload(dp, hp, s));
+  return upload(ds, st, s);
 }
 
 // Image-space points sorted by the 8^3 home tile of their first tap, then by
 // cell (the order of the home-tile spread, spread_home.cu), with the first
 // sorted index of every home tile, and the super-tile scratch.
-nrsense_status build_home_set(nrsense_plan_s* p, const std::vector<HostPoint>& pts,
-                              cudaStream_t s) {
+nrsense_status build_home_set(nrsense_plan_s* p, cudaStream_t s) {
   const Geo& g = p->geo;
+  if (p->home_scratch != nullptr) return NRSENSE_OK;  // built
   HomeSet& hs = p->ihome;
   hs.nt0 = (g.g0 + 7) / 8;
   hs.nt1 = (g.g1 + 7) / 8;
@@ -423,42 +559,7 @@ nrsense_status build_home_set(nrsense_plan_s* p, const std::vector<HostPoint>& p
   hs.ns0 = (g.g0 + 15) / 16;
   hs.ns1 = (g.g1 + 15) / 16;
   hs.ns2 = (g.g2 + 15) / 16;
-  const long long ntl = (long long)hs.nt0 * hs.nt1 * hs.nt2;
-  const long long npts = (long long)pts.size();
-  // (key << 32 | index): sorting by it is stable in the input order
-  std::vector<uint64_t> ko(npts);
-  std::vector<int32_t> tstart(ntl + 1, 0);
-  for (long long i = 0; i < npts; ++i) {
-    const HostPoint& h = pts[i];
-    const long long t = ((long long)(h.b[0] >> 3) * hs.nt1 + (h.b[1] >> 3)) * hs.nt2 + (h.b[2] >> 3);
-    const int cell = (((h.b[0] & 7) * 8) + (h.b[1] & 7)) * 8 + (h.b[2] & 7);
-    ko[i] = (uint64_t(t * 512 + cell) << 32) | uint64_t(i);
-    tstart[t + 1]++;
-  }
-  std::sort(ko.begin(), ko.end());
-  for (long long t = 0; t < ntl; ++t) tstart[t + 1] += tstart[t];
-  std::vector<float4> qs(std::max<long long>(npts, 1));
-  std::vector<int32_t> perm(std::max<long long>(npts, 1));
-  for (long long k = 0; k < npts; ++k) {
-    const HostPoint& h = pts[ko[k] & 0xffffffffu];
-    const uint32_t packed = pack_base(h.b[0], h.b[1], h.b[2]);
-    float w;
-    std::memcpy(&w, &packed, sizeof(w));
-    qs[k] = make_float4(h.f[0], h.f[1], h.f[2], w);
-    perm[k] = h.row;
-  }
-  std::vector<uint64_t>().swap(ko);
-  float4* dq = nullptr;
-  int32_t *dp = nullptr, *dt = nullptr;
-  NRS_TRY(dev_alloc_n(p, &dq, (long long)qs.size()));
-  NRS_TRY(dev_alloc_n(p, &dp, (long long)perm.size()));
-  NRS_TRY(dev_alloc_n(p, &dt, ntl + 1));
-  NRS_TRY(upload(dq, qs, s));
-  NRS_TRY(upload(dp, perm, s));
-  NRS_TRY(upload(dt, tstart, s));
-  hs.qs = dq;
-  hs.perm = dp;
-  hs.tstart = dt;
+  NRS_TRY(sorted_image_points(p, 3, true, &hs.qs, &hs.perm, &hs.tstart, s));
   // per axis and coordinate: the super-tiles whose 3-point-padded extents
   // cover it (directly or wrapped around the periodic grid), increasing
   const int gsz[3] = {g.g0, g.g1, g.g2}, nsz[3] = {hs.ns0, hs.ns1, hs.ns2};
@@ -483,57 +584,20 @@ nrsense_status build_home_set(nrsense_plan_s* p, const std::vector<HostPoint>& p
     if (cudaStreamSynchronize(s) != cudaSuccess) return NRSENSE_ERR_CUDA;
     *cov[a] = dtab;
   }
-  NRS_TRY(dev_alloc_n(p, &p->home_scratch, home_scratch_elems(hs)));
   if (configure_home_kernels() != cudaSuccess) return NRSENSE_ERR_CUDA;
-  p->home_ok = true;
-  // host vectors are freed on return: wait for the uploads
-  if (cudaStreamSynchronize(s) != cudaSuccess) return NRSENSE_ERR_CUDA;
-  return NRSENSE_OK;
+  return dev_alloc_n(p, &p->home_scratch, home_scratch_elems(hs));
 }
 
 // Image-space points sorted by the 4^3 block of their first tap (stable), with
 // the first sorted index of every block (spread_rows.cu).
-nrsense_status build_row_set(nrsense_plan_s* p, const std::vector<HostPoint>& pts, cudaStream_t s) {
+nrsense_status build_row_set(nrsense_plan_s* p, cudaStream_t s) {
   const Geo& g = p->geo;
   RowSet& rs = p->irows;
   rs.nb0 = g.g0 / 4;
   rs.nb1 = g.g1 / 4;
   rs.nb2 = g.g2 / 4;
-  const size_t nblk = (size_t)rs.nb0 * rs.nb1 * rs.nb2, n = pts.size();
-  auto block = [&](const HostPoint& h) {
-    return ((size_t)(h.b[0] >> 2) * rs.nb1 + (h.b[1] >> 2)) * rs.nb2 + (h.b[2] >> 2);
-  };
-  std::vector<int32_t> start(nblk + 1, 0), at(nblk);
-  for (const HostPoint& h : pts) start[block(h) + 1]++;
-  for (size_t b = 0; b < nblk; ++b) start[b + 1] += start[b];
-  std::copy(start.begin(), start.end() - 1, at.begin());
-  std::vector<float4> qs(std::max<size_t>(n, 1));
-  std::vector<int32_t> perm(std::max<size_t>(n, 1));
-  for (const HostPoint& h : pts) {
-    const size_t k = size_t(at[block(h)]++);
-    const uint32_t packed = pack_base(h.b[0], h.b[1], h.b[2]);
-    float w;
-    std::memcpy(&w, &packed, sizeof(w));
-    qs[k] = make_float4(h.f[0], h.f[1], h.f[2], w);
-    perm[k] = h.row;
-  }
-  float4* dq = nullptr;
-  int32_t *dp = nullptr, *ds = nullptr;
-  NRS_TRY(dev_alloc_n(p, &dq, (long long)qs.size()));
-  NRS_TRY(dev_alloc_n(p, &dp, (long long)perm.size()));
-  NRS_TRY(dev_alloc_n(p, &ds, (long long)start.size()));
-  NRS_TRY(upload(dq, qs, s));
-  NRS_TRY(upload(dp, perm, s));
-  NRS_TRY(upload(ds, start, s));
-  rs.qs = dq;
-  rs.perm = dp;
-  rs.start = ds;
+  NRS_TRY(sorted_image_points(p, 2, false, &rs.qs, &rs.perm, &rs.start, s));
   p->rows_ok = true;
-  // rows against home tiles, points per grid value: 1/8 (one phase at sigma 2)
-  // 0.695 against 1.08 ms at 384^3, 1/4 (two phases) 0.40 against 0.40 ms at
-  // 256^3, 1/2 0.76 against 0.59: the home tiles' fixed cost per tile
-  // (accumulators, merge, rims) against the rows' four visits per point
-  p->rows_sparse = p->W == 4 && 6 * (long long)n <= g.ngrid;
   return NRSENSE_OK;
 }
 
@@ -545,7 +609,7 @@ nrsense_status ensure_scratch(nrsense_plan_s* p) {
     return (long long)ps.tp.t0 * ps.tp.t1 * ps.tp.t2;
   };
   if (!p->identity_warp) need = std::max(need, (long long)p->ipts.n_slots * tile_pts(p->ipts));
-  if (p->C > 0) {
+  if (p->C > 0 && !p->kpts.empty()) {
     const int cc = spread_coil_chunk(p->C);
     const int chunks = (p->C + cc - 1) / cc;
     for (int j0 = 0; j0 < p->P; j0 += p->phase_chunk) {
@@ -561,6 +625,16 @@ nrsense_status ensure_scratch(nrsense_plan_s* p) {
   NRS_TRY(dev_alloc_n(p, &p->b_scratch, need));
   p->scratch_elems = need;
   return NRSENSE_OK;
+}
+
+// halo lists of the displaced voxels (the spread over per-tile lists)
+nrsense_status build_image_lists(nrsense_plan_s* p, cudaStream_t s) {
+  if (p->ipts.qs != nullptr) return NRSENSE_OK;
+  std::vector<HostPoint> pts;
+  NRS_TRY(host_image_points(p, pts, s));
+  NRS_TRY(build_pointset(p, pts, &p->ipts, p->itiles, nullptr, /*interp=*/false, kSpreadMaxItemImage,
+                         s));
+  return ensure_scratch(p);
 }
 
 nrsense_status cufft_check(cufftResult r) {
@@ -687,39 +761,25 @@ nrsense_status create_impl(nrsense_plan_s* p, const nrsense_desc* desc, const in
     if (cudaMemcpyAsync(p->disp, disp, size_t(nd) * sizeof(float), cudaMemcpyDeviceToDevice, s) !=
         cudaSuccess)
       return NRSENSE_ERR_CUDA;
-    std::vector<float> hd(nd);
-    if (cudaMemcpyAsync(hd.data(), disp, size_t(nd) * sizeof(float), cudaMemcpyDeviceToHost, s) !=
-            cudaSuccess ||
-        cudaStreamSynchronize(s) != cudaSuccess)
-      return NRSENSE_ERR_CUDA;
-    for (long long i = 0; i < nd; ++i)
-      if (!std::isfinite(hd[i]) || std::fabs(hd[i]) > 1e6f) return NRSENSE_ERR_ARG;
-    std::vector<HostPoint> pts((size_t)(p->P * g.nvox));
-    const int gs[3] = {g.g0, g.g1, g.g2};
-    for (int j = 0; j < p->P; ++j) {
-      const float* dj = hd.data() + (long long)j * 3 * g.nvox;
-      for (long long v = 0; v < g.nvox; ++v) {
-        const int i2 = int(v % g.n2);
-        const int i1 = int((v / g.n2) % g.n1);
-        const int i0 = int(v / ((long long)g.n1 * g.n2));
-        const int ii[3] = {i0, i1, i2};
-        HostPoint& h = pts[(size_t)(j * g.nvox + v)];
-        for (int a = 0; a < 3; ++a) {
-          // q = sigma * (n + d) = sigma*n + sigma*d in FP64 (sigma*n exact)
-          const double q = sigma * double(ii[a]) + sigma * double(dj[a * g.nvox + v]);
-          decompose(q, gs[a], p->W, &h.b[a], &h.f[a]);
-        }
-        h.row = int32_t(j * g.nvox + v);
-      }
-    }
-    NRS_TRY(build_pointset(p, pts, &p->ipts, itiles, nullptr, /*interp=*/false,
-                           kSpreadMaxItemImage, s));
-    if (!p->comp_spread && !p->grid_bf16 && g.g0 % 4 == 0 && g.g1 % 4 == 0 && g.g2 % 4 == 0)
-      NRS_TRY(build_row_set(p, pts, s));
-    // home-tile spread (W = 4, plain FP32 accumulation); the default where built
-    if (p->W == 4 && !p->comp_spread) {
-      NRS_TRY(build_home_set(p, pts, s));
-      p->spread_image_variant = kSpreadHome;
+    if (cudaStreamSynchronize(s) != cudaSuccess) return NRSENSE_ERR_CUDA;
+    p->ipts.tp = itiles;
+    // the point order of the spread that the plan starts with (the others are
+    // built when a tuning choice needs them).  Rows against home tiles, points per
+    // grid value: 1/8 (one phase at sigma 2) 0.695 against 1.08 ms at 384^3, 1/4
+    // (two phases) 0.40 against 0.40 ms at 256^3, 1/2 0.76 against 0.59: the home
+    // tiles' fixed cost per tile (accumulators, merge, rims) against the rows' four
+    // visits per point
+    const bool rows = !p->comp_spread && !p->grid_bf16 && g.g0 % 4 == 0 && g.g1 % 4 == 0 &&
+                      g.g2 % 4 == 0;
+    p->rows_sparse = rows && p->W == 4 && 6 * p->P * g.nvox <= g.ngrid;
+    p->home_ok = p->W == 4 && !p->comp_spread;
+    if (p->home_ok) p->spread_image_variant = kSpreadHome;
+    if (rows && (p->W != 4 || p->rows_sparse)) {
+      NRS_TRY(build_row_set(p, s));
+    } else if (p->home_ok) {
+      NRS_TRY(build_home_set(p, s));
+    } else {
+      NRS_TRY(build_image_lists(p, s));
     }
   }
 
@@ -750,7 +810,8 @@ nrsense_status create_impl(nrsense_plan_s* p, const nrsense_desc* desc, const in
     p->kpts.resize(p->P);
     const int gs[3] = {g.g0, g.g1, g.g2};
     std::vector<std::vector<HostPoint>> all((size_t)p->P);
-    for (int j = 0; j < p->P; ++j) {
+    std::vector<std::vector<char>> touch((size_t)p->P);
+    NRS_TRY(for_phases(p->P, [&](int j) -> nrsense_status {
       std::vector<HostPoint>& pts = all[(size_t)j];
       pts.resize((size_t)p->M[j]);
       for (long long i = 0; i < p->M[j]; ++i) {
@@ -764,11 +825,15 @@ nrsense_status create_impl(nrsense_plan_s* p, const nrsense_desc* desc, const in
         }
         h.row = int32_t(i);
       }
-    }
+      touch[(size_t)j].assign((size_t)ktiles.ntiles, 0);
+      mark_touched_tiles(p, ktiles, pts, touch[(size_t)j]);
+      return NRSENSE_OK;
+    }));
     // all phases share one spread target: each phase writes every tile that
     // any phase occupies (zeros where it has no points), the rest stay zero
     std::vector<char> uni((size_t)ktiles.ntiles, 0);
-    for (int j = 0; j < p->P; ++j) mark_touched_tiles(p, ktiles, all[(size_t)j], uni);
+    for (const std::vector<char>& t : touch)
+      for (size_t k = 0; k < uni.size(); ++k) uni[k] |= t[k];
     long long nuni = 0;
     for (char u : uni) nuni += u != 0;
     p->kuni_fraction = double(nuni) / double(uni.size());
@@ -798,10 +863,16 @@ nrsense_status create_impl(nrsense_plan_s* p, const nrsense_desc* desc, const in
       NRS_TRY(dev_alloc_n(p, &p->kanymask, (long long)am.size()));
       NRS_TRY(upload(p->kanymask, am, s));
     }
-    for (int j = 0; j < p->P; ++j) {
-      NRS_TRY(build_pointset(p, all[(size_t)j], &p->kpts[j], ktiles, &uni, /*interp=*/true,
-                             p->spread_max_item, s));
+    std::vector<HostSet> sets((size_t)p->P);
+    NRS_TRY(for_phases(p->P, [&](int j) -> nrsense_status {
+      const nrsense_status st = compute_pointset(g, p->W, all[(size_t)j], ktiles, &uni, /*interp=*/true,
+                                                 p->spread_max_item, &sets[(size_t)j]);
       std::vector<HostPoint>().swap(all[(size_t)j]);
+      return st;
+    }));
+    for (int j = 0; j < p->P; ++j) {
+      NRS_TRY(upload_pointset(p, sets[(size_t)j], &p->kpts[j], s));
+      sets[(size_t)j] = HostSet{};
     }
     p->kunion.swap(uni);
   }
@@ -949,6 +1020,17 @@ void release(nrsense_plan_s* p) {
 }  // namespace
 
 namespace nrs {
+
+nrsense_status ensure_image_sets(nrsense_plan_s* p, bool lists, bool home, cudaStream_t s) {
+  if (p->identity_warp) return NRSENSE_OK;
+  try {
+    if (lists) NRS_TRY(build_image_lists(p, s));
+    if (home) NRS_TRY(build_home_set(p, s));
+  } catch (const std::bad_alloc&) {
+    return NRSENSE_ERR_OOM;
+  }
+  return NRSENSE_OK;
+}
 
 nrsense_status retile_kspace(nrsense_plan_s* p, int max_item, cudaStream_t s) {
   p->epoch += 1;  // point-set buffers are rebuilt

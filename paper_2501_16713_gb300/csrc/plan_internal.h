@@ -103,7 +103,7 @@ struct nrsense_plan_s {
   nrs::RowSet irows{};              // the same, sorted by 4^3 block (row spread)
   bool rows_ok = false;             // irows built (grids of a multiple of 4, plain FP32)
   bool rows_sparse = false;         // rows_ok, W = 4 and few enough points for the row spread
-  bool home_ok = false;             // ihome built (W = 4, not compensated)
+  bool home_ok = false;             // ihome applies (W = 4, not compensated); built when used
   // image-space interpolation over super-tiles (autotuned; a thread per voxel
   // until then: 0.324 against 0.414 ms at 192^3 with one phase, 0.300 against
   // 0.309 at 128^3 with four, 0.0067 against 0.0148 at 32^3)
@@ -393,6 +393,12 @@ int launch_mixed_image_up(const Geo& g, const MixAxis* ax, const float* deapod,
 int launch_mixed_image_down(const Geo& g, const MixAxis* ax, const float* deapod,
                             const nrsense_c64* u, void* t2, void* t1, nrsense_c64* x,
                             cudaStream_t s);
+// device sort of the displaced voxels (plan_image.cu)
+nrsense_status sort_image_points(const Geo& g, int W, double sigma, long long n, const float* disp,
+                                 int shift, bool cells, float4* qs, int32_t* perm, int32_t* start,
+                                 bool* bad, bool* done, cudaStream_t s);
+// build the image-space halo lists / home tiles where not built yet (plan.cu)
+nrsense_status ensure_image_sets(nrsense_plan_s* p, bool lists, bool home, cudaStream_t s);
 // rebuild the k-space spreading work items of every phase with at most
 // max_item list entries per item (plan.cu; the lists of split tiles are
 // re-dealt, the sorted points stay) and grow the split-tile scratch if needed
