@@ -550,7 +550,8 @@ nrsense_status nrsense_symmetric_eigen(int32_t m, const double* a_host, double* 
  * nrsense_plan_set_tuning applies stored choices (e.g. a cache keyed by the
  * geometry).  Both change only speed: every choice computes the same values
  * (bitwise, except the tensor-core spread and the pruned transforms, which
- * agree to FP32 rounding).
+ * agree to FP32 rounding).  set_tuning builds the image-space point order that a choice
+ * needs where the plan does not have it yet (device memory; synchronises).
  * Errors: ERR_ARG (null, reps outside 1..100, unknown choice), ERR_CUDA.
  */
 #define NRSENSE_TUNE_SPREAD_REGISTER      1  /* register accumulation, CTA per tile */
@@ -559,7 +560,8 @@ nrsense_status nrsense_symmetric_eigen(int32_t m, const double* a_host, double* 
 #define NRSENSE_TUNE_SPREAD_MMA           4  /* tensor-core accumulation (TF32 split in three
                                                 products), a warp per tile plane or per 4^3
                                                 sub-block, 8-coil chunks
-                                                (fewer coils: as REGISTER_WARP); within FP32
+                                                (four coils and fewer: FP32 FMAs by sub-blocks;
+                                                BF16 grids: as REGISTER_WARP); within FP32
                                                 rounding of, not bitwise equal to, the others */
 typedef struct {
   int32_t spread_variant;  /* NRSENSE_TUNE_SPREAD_* */
@@ -572,13 +574,16 @@ typedef struct {
   int32_t spread_image_warp;   /* image-space spread: 0 CTA per tile, 1 CTA per plane pair
                                   (both over per-tile halo lists), 2 home tiles (every displaced
                                   voxel spread once by the warp of the 8^3 tile holding its first
-                                  tap, super-tile rims summed by a second kernel; W = 4 and not
-                                  compensated; set_tuning rejects 2 elsewhere) */
+                                  tap, super-tile rims summed by a second kernel; on grids with
+                                  at most a point per six values, rows of 4^3 blocks instead;
+                                  W = 4 and not compensated; set_tuning rejects 2 elsewhere) */
   double  spread_image_ms[3];  /* measured: CTA per tile, CTA per plane pair, home tiles
                                   (-1: n/a) */
   int32_t fft_pruned;          /* 1: own pruned coil-grid transforms with the coil fan-out and
                                   combination fused (sigma 2, power-of-two grid sizes 32..256,
-                                  FP32 grids); 0: cuFFT plus the fan-out / combination kernels */
+                                  FP32 grids); 0: cuFFT plus the fan-out / combination kernels
+                                  (grids of other sizes take the mixed-radix passes either way,
+                                  where their prime factors are at most 13) */
   double  fft_ms[2];           /* measured forward + adjoint of the first phase chunk:
                                   cuFFT path, pruned path (-1: not available) */
   double  spread_mma_ms;       /* measured tensor-core spread, best geometry and warps per CTA
@@ -608,7 +613,8 @@ typedef struct {
                                   zero-padding / cropping fused into the x passes; sigma 2,
                                   power-of-two grid sizes 32..256, not with the compensated
                                   precision; set_tuning rejects 1 elsewhere), 0 cuFFT plus the
-                                  deapodization kernels */
+                                  deapodization kernels (grids of other sizes: the mixed-radix
+                                  passes either way, as above) */
   double  image_fft_ms[2];     /* measured forward + adjoint G^3 transforms with their
                                   deapodization: cuFFT path, pruned path (-1: n/a) */
 } nrsense_tuning;

@@ -19,9 +19,9 @@
 // z passes close behind (at 384 points fwd_y 57 %, fwd_z 49 %, inv_z 51 % of the
 // DRAM rate with 41-46 instructions per element).  16 lanes per CTA make 128-byte
 // rows of every access.  Replaced cuFFT with separate fan-out, combination,
-// padding and N^3 kernels: 16 coil grids of 384^3 forward 8.55 -> 3.38 ms, 16 of
+// padding and N^3 kernels: 16 coil grids of 384^3 forward 8.55 -> 3.06 ms, 16 of
 // 512^3 adjoint 16.9 -> 8.2 ms, three phases of 5 grids of 168 x 120 x 264 both
-// ways 1.94 -> 0.81 ms, T's 384^3 image grid 0.81 -> 0.41 ms a direction, 64^3
+// ways 1.94 -> 0.81 ms, T's 384^3 image grid 0.81 -> 0.31 ms a direction, 64^3
 // images 0.078 -> 0.045 ms and 32^3 ones 0.060 -> 0.030 ms for T and T^H.
 #pragma once
 
@@ -358,8 +358,10 @@ inline int steps_of(const GeneralAxis& a, bool image, int* nb) {
 // to bring the warps: 256 where that leaves at most a quarter of the thread turns
 // over the steps idle (384-point coil passes, 16 x (16, 24) butterflies: 3.06 ms for
 // 16 grids against 3.38 with 128 threads and none idle), else the largest multiple of
-// 32 that leaves at most 15 % idle (T's 384-point passes with 64 threads, none idle
-// and 6 warps per SM: 0.41 ms; with 128: 0.32), else the one that leaves the fewest.
+// 32 that leaves at most 15 % idle, else the one that leaves the fewest.  T's
+// 384-point passes: 64 threads, none idle and 6 warps per SM, 0.41 ms; 128, 0.32;
+// 256, 0.31.  With 25 % allowed below 256 threads too the N = 64 passes went from
+// 0.26 to 0.28 ms and run-time radices (168 x 120 x 264) from 0.81 to 0.89.
 template <class AX>
 int threads_for(const AX& ax, bool image) {
   int nb[6], work = 0;
