@@ -13,7 +13,8 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
-#include <system_error>
+#include <exception>
+#include <new>
 #include <thread>
 #include <vector>
 
@@ -441,7 +442,7 @@ nrsense_status for_phases(int n, F&& f) {
     for (int j = k; j < n; j += nt) {
       try {
         st[(size_t)j] = f(j);
-      } catch (const std::bad_alloc&) {
+      } catch (const std::exception&) {
         st[(size_t)j] = NRSENSE_ERR_OOM;
       }
     }
@@ -449,9 +450,10 @@ nrsense_status for_phases(int n, F&& f) {
   std::vector<std::thread> pool;
   int started = 1;
   try {
+    pool.reserve((size_t)nt);
     for (; started < nt; ++started) pool.emplace_back(work, started);
-  } catch (const std::system_error&) {
-    // no more threads: this one takes the rest
+  } catch (const std::exception&) {
+    // no more threads, or no memory for their state: this one takes the rest
   }
   work(0);
   for (std::thread& t : pool) t.join();
