@@ -636,6 +636,7 @@ nrsense_status nrsense_plan_autotune(nrsense_plan_t p, int32_t reps, nrsense_tun
   out->spread_mma_wpc = 0;
   out->spread_mma_cube = 0;
   out->spread_mma_geo_ms[0] = out->spread_mma_geo_ms[1] = -1.0;
+  double pick = -1.0;  // time of the tensor-core (or sub-block) candidate taken
   if (mma_ok) {
     const int wpcs[3] = {1, 2, 4};
     for (int cube = 0; cube < 2; ++cube) {
@@ -650,8 +651,13 @@ nrsense_status nrsense_plan_autotune(nrsense_plan_t p, int32_t reps, nrsense_tun
         if (ms < 0.0) continue;
         double& geo_ms = out->spread_mma_geo_ms[cube];
         if (geo_ms < 0.0 || ms < geo_ms) geo_ms = ms;
-        if (out->spread_mma_ms < 0.0 || ms < out->spread_mma_ms) {
-          out->spread_mma_ms = ms;
+        if (out->spread_mma_ms < 0.0 || ms < out->spread_mma_ms) out->spread_mma_ms = ms;
+        // FP32 grids: the sub-block kernel where it can run, whose sums are
+        // FP32-accurate (the plane kernel lets the tensor core truncate its
+        // running sum, a few 1e-6, and does 29 % more products)
+        const bool exact = cube == 1 && !p->grid_bf16;
+        if (pick < 0.0 || ms < pick || (exact && out->spread_mma_cube == 0)) {
+          pick = ms;
           out->spread_mma_wpc = wpcs[k];
           out->spread_mma_cube = cube;
         }
@@ -664,6 +670,7 @@ nrsense_status nrsense_plan_autotune(nrsense_plan_t p, int32_t reps, nrsense_tun
                                    false, spread_mma_variant(1, false), p->b_scratch, p->d_status, s);
     });
     out->spread_mma_wpc = 1;
+    pick = out->spread_mma_ms;
   }
   const int chunks[2] = {8, 4};
   const bool saved_tma = p->interp_tma;
@@ -728,7 +735,7 @@ nrsense_status nrsense_plan_autotune(nrsense_plan_t p, int32_t reps, nrsense_tun
     for (int k = 1; k < 3; ++k)
       if (out->spread_ms[k] < out->spread_ms[bk]) bk = k;
     p->spread_variant = variants[bk];
-    if ((mma_ok || few_ok) && out->spread_mma_ms >= 0.0 && out->spread_mma_ms < out->spread_ms[bk])
+    if ((mma_ok || few_ok) && pick >= 0.0 && pick < out->spread_ms[bk])
       p->spread_variant = spread_mma_variant(out->spread_mma_wpc, out->spread_mma_cube == 1);
   }
   // fastest interpolation: staging (per value / TMA) x coils per CTA (8 / 4; TMA also 2)

@@ -580,15 +580,17 @@ __global__ void __launch_bounds__(32 * WPC, WPC == 4 ? 5 : 16 / WPC) spread_coil
 // fall by 29 %.  Rows m = 16 z + 4 y + x of the sub-block (z, y, x in 0..3):
 // lane (g, q) holds x = g % 4 with y = g / 4 (row g) and y + 2 (row g + 8) for
 // every m-tile z.  Columns and the TF32 split are those of the plane kernel.
-// EXACT: every k-step's eight points are summed from a zero accumulator, small
-// terms first, and added to the sums by one rounded FP32 addition (16 more
-// additions and 8 more registers per k-step): the tensor core truncates its
-// running sum, which over a dense sub-block's hundreds of steps costs a few 1e-6.
+// EXACT (FP32 grids): every k-step's eight points are summed from a zero
+// accumulator, small terms first, and added to the sums by one rounded FP32
+// addition (16 more additions per k-step): the tensor core truncates its running
+// sum, which over a dense sub-block's hundreds of steps costs a few 1e-6, and
+// which a CG solve then carries on (64^3, 8 coils, six iterations: 2e-6 to 1e-5).
 // 256^3, 16 coils, 3 M samples: 4.20 against 4.01 ms, error of the adjoint on
-// positive data 2.8e-7 against 5.3e-6 (register kernel 6.50 ms, 2.9e-7).
+// positive data 2.8e-7 against 5.3e-6 (register kernel 6.50 ms, 2.9e-7).  E at
+// 128^3, 8 coils, 4 phases: 8.18 against 8.15 ms (8.28 at 24 warps per SM).
 // A k-step skips the m-tiles none of its eight points reaches (the runs are in
 // first-tap z order, so neighbouring points mostly share their z planes).  The
-// launch bound of 28 warps per SM holds the kernel at 72 registers; with one
+// launch bound of 28 warps per SM holds the W = 4 kernel at 72 registers; with one
 // warp per CTA (the usual choice) a CTA's slot frees as soon as its sub-block
 // is done, whatever the other sub-blocks' point counts.
 template <int W>
@@ -609,7 +611,7 @@ __device__ __forceinline__ void put_taps(float* dst, const float (&w)[W]) {
 }
 
 template <typename GT, int WPC, int W, bool EXACT>
-__global__ void __launch_bounds__(32 * WPC, (EXACT ? 24 : 28) / WPC) spread_coils_cube_kernel(
+__global__ void __launch_bounds__(32 * WPC, (W == 6 ? 24 : 28) / WPC) spread_coils_cube_kernel(
     Geo g, KernelCoefs kc, int C, TilePlan tp, PhaseTable pt, const float2* __restrict__ vals,
     GT* __restrict__ grids, float2* __restrict__ scratch) {
   constexpr int CC = 8, T = 8, B = 32;
@@ -1248,27 +1250,29 @@ int launch_reduce(const Geo& g, int C, const TilePlan& tp, const PhaseTable& pt,
   return 1;
 }
 
-// the sub-block spread over 8-coil chunks, wpc (1, 2 or 4) sub-blocks per CTA
+// the sub-block spread over 8-coil chunks, wpc (1, 2 or 4) sub-blocks per CTA; BF16
+// grids keep the tensor core's running sum, whose error their rounding covers
 template <typename GT, int W>
 void launch_cube(const Geo& g, const KernelCoefs& kc, int C, const TilePlan& tp,
                  const PhaseTable& pt, const float2* vals, GT* grids, float2* scratch, int wpc,
-                 bool exact, cudaStream_t s) {
+                 cudaStream_t s) {
+  constexpr bool kExact = sizeof(GT) == 8;
   const unsigned blocks = 8u * pt.item0[pt.nphase];
   const int chunks = (C + 7) / 8;
-  if (exact || W != 4)
-    spread_coils_cube_kernel<GT, 1, W, true><<<dim3(blocks, chunks), 32, 0, s>>>(
-        g, kc, C, tp, pt, vals, grids, scratch);
-  else if constexpr (W == 4) {
-    if (wpc == 4)
-      spread_coils_cube_kernel<GT, 4, W, false><<<dim3(blocks / 4, chunks), 128, 0, s>>>(
+  if constexpr (W == 4) {
+    if (wpc == 4) {
+      spread_coils_cube_kernel<GT, 4, W, kExact><<<dim3(blocks / 4, chunks), 128, 0, s>>>(
           g, kc, C, tp, pt, vals, grids, scratch);
-    else if (wpc == 2)
-      spread_coils_cube_kernel<GT, 2, W, false><<<dim3(blocks / 2, chunks), 64, 0, s>>>(
+      return;
+    }
+    if (wpc == 2) {
+      spread_coils_cube_kernel<GT, 2, W, kExact><<<dim3(blocks / 2, chunks), 64, 0, s>>>(
           g, kc, C, tp, pt, vals, grids, scratch);
-    else
-      spread_coils_cube_kernel<GT, 1, W, false><<<dim3(blocks, chunks), 32, 0, s>>>(
-          g, kc, C, tp, pt, vals, grids, scratch);
+      return;
+    }
   }
+  spread_coils_cube_kernel<GT, 1, W, kExact><<<dim3(blocks, chunks), 32, 0, s>>>(
+      g, kc, C, tp, pt, vals, grids, scratch);
 }
 
 template <int CC, int W>
@@ -1297,8 +1301,7 @@ int dispatch_coils(const Geo& g, const KernelCoefs& kc, int C, const TilePlan& t
     if constexpr (CC < 8 && sizeof(GT) == 8) launch_few<CC, 4>(g, kc, C, tp, pt, vals, grids, scratch, s);
   } else if (CC == 8 && ((variant == kSpreadMMA && mma_cube) || variant == kSpreadCubeExact) &&
              pt.clist[0] != nullptr) {
-    launch_cube<GT, 4>(g, kc, C, tp, pt, vals, grids, scratch, mma_wpc,
-                       variant == kSpreadCubeExact, s);
+    launch_cube<GT, 4>(g, kc, C, tp, pt, vals, grids, scratch, mma_wpc, s);
   } else if (variant == kSpreadMMA && CC == 8) {
     const unsigned planes = 8u * pt.item0[pt.nphase];
     if (mma_wpc == 4)
@@ -1360,7 +1363,7 @@ int spread_multi(const Geo& g, int W, const KernelCoefs& kc, int C, const TilePl
         launch_few<4, 6>(g, kc, C, tp, pt, v, gr, sc, s);
         return 1 + launch_reduce<8, 4, GT>(g, C, tp, pt, chunks, gr, sc, s);
       }
-      launch_cube<GT, 6>(g, kc, C, tp, pt, v, gr, sc, 1, true, s);
+      launch_cube<GT, 6>(g, kc, C, tp, pt, v, gr, sc, 1, s);
       return 1 + launch_reduce<8, 8, GT>(g, C, tp, pt, chunks, gr, sc, s);
     }
   }

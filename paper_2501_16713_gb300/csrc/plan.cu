@@ -981,9 +981,7 @@ nrsense_status create_impl(nrsense_plan_s* p, const nrsense_desc* desc, const in
     // samples: 4.20 ms against 6.50 of the register kernel, the adjoint's error
     // 2.6e-7 against 2.7e-7), or by FMAs (2 coils at 64^3, 100 k samples: 0.091 against
     // 0.137 ms; with 3 and 4 coils the register kernel is the faster one on dense
-    // samples, 0.495 against 0.634 ms at 128^3, and the tuner times both).  The tuner's tensor-core
-    // candidate lets the tensor core accumulate, 4 % faster, with errors of a few
-    // 1e-6.  BF16 grids keep the register kernel and its exact summation order.
+    // samples, 0.495 against 0.634 ms at 128^3, and the tuner times both).  BF16 grids keep the register kernel and its exact summation order.
     if (p->tma_ok) {
       p->interp_tma = true;
       p->interp_coils = p->C <= 2 ? 2 : 4;
