@@ -585,7 +585,8 @@ __global__ void __launch_bounds__(32 * WPC, WPC == 4 ? 5 : 16 / WPC) spread_coil
 // addition (16 more additions per k-step): the tensor core truncates its running
 // sum, which over a dense sub-block's hundreds of steps costs a few 1e-6, and
 // which a CG solve then carries on (64^3, 8 coils, six iterations: 2e-6 to 1e-5).
-// 256^3, 16 coils, 3 M samples: 4.20 against 4.01 ms, error of the adjoint on
+// 256^3, 16 coils, 3 M samples: 4.20 (at 24 warps per SM; the whole adjoint 12.53 ->
+// 12.21 ms with 28) against 4.01 ms, error of the adjoint on
 // positive data 2.8e-7 against 5.3e-6 (register kernel 6.50 ms, 2.9e-7).  E at
 // 128^3, 8 coils, 4 phases: 8.18 against 8.15 ms (8.28 at 24 warps per SM).
 // A k-step skips the m-tiles none of its eight points reaches (the runs are in

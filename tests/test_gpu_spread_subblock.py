@@ -70,3 +70,24 @@ def test_density_compensation_matches_oracle(shape, width, samples):
     ref, _ = OM.dcf_pipe_menon(O.Geometry(shape, width=width), c["coords"][0], 4)
     assert rel_l2(w, ref) < TOL_FP32
     plan.close()
+
+
+@pytest.mark.parametrize("wpc,coils", [(1, 8), (2, 6), (4, 11)])
+def test_tuned_sub_blocks_sum_in_fp32(wpc, coils):
+    """Positive data, where a truncated running sum drifts one way.  Weights, sums, transform
+    and coil combination are FP32 steps of at most some 2.5e-7 each: 1e-6 together."""
+    import ctypes
+    from paper_2501_16713_gb300.nrsense import Tuning
+    shape = (16, 14, 18)
+    c = synth.small_case(shape, coils, 1, [40000], seed=104)
+    plan = make_plan(c, shape, identity_warp=True)
+    t = Tuning()
+    t.spread_variant, t.interp_coils, t.interp_tma = 4, 8, 0
+    t.spread_mma_wpc, t.spread_mma_cube = wpc, 1
+    assert plan.lib.nrsense_plan_set_tuning(plan._h, ctypes.byref(t)) == 0
+    y = (1.0 + 0.1 * crandn(np.random.default_rng(105), (40000, coils))).astype(np.complex64)
+    ref = O.stacked_adjoint(O.Geometry(shape), [y.astype(np.complex128)], [None], c["smaps"], c["coords"])
+    err = rel_l2(plan.adjoint(to_dev(y)).cpu().numpy(), ref)
+    print(wpc, coils, "adjoint rel L2 %.2e" % err)
+    assert err < 1e-6
+    plan.close()
