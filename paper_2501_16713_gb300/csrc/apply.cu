@@ -261,7 +261,7 @@ nrsense_status warp_adjoint(nrsense_plan_s* p, const nrsense_c64* m, nrsense_c64
   } else {
     const PhaseTable t = image_table(p);
     STAGE(SPREAD_IMAGE, launch_spread(g, p->W, p->kc, 1, p->itiles, t, m, p->b_ugrid, false,
-                                      p->comp_spread, p->spread_image_variant, p->b_scratch,
+                                      p->comp_spread, p->spread_image_variant, p->image_scratch,
                                       p->d_status, s));
   }
   NRS_TRY(launched());
@@ -526,7 +526,8 @@ nrsense_status nrsense_plan_autotune(nrsense_plan_t p, int32_t reps, nrsense_tun
                                             p->home_scratch, s);
         else
           p->launches += launch_spread(g, p->W, p->kc, 1, p->itiles, tim, p->b_m, p->b_ugrid,
-                                       false, p->comp_spread, iv[k], p->b_scratch, p->d_status, s);
+                                       false, p->comp_spread, iv[k], p->image_scratch, p->d_status,
+                                       s);
       };
       run();
       cudaEventRecord(a, s);

@@ -27,16 +27,21 @@ using namespace nrs;
 
 namespace {
 
-// Host-side fault injection for the error paths (NRSENSE_FAULT=alloc|cufft|upload).
-bool fault_requested(const char* what) {
+// Host-side fault injection for the error paths (NRSENSE_FAULT=alloc|cufft|upload;
+// alloc:N: allocations of a plan that holds N already).
+bool fault_requested(const char* what, const nrsense_plan_s* p = nullptr) {
   const char* f = std::getenv("NRSENSE_FAULT");
-  return f != nullptr && std::strcmp(f, what) == 0;
+  if (f == nullptr) return false;
+  const size_t n = std::strlen(what);
+  if (std::strncmp(f, what, n) != 0) return false;
+  return f[n] == '\0' || (f[n] == ':' && p != nullptr &&
+                          p->allocations.size() >= size_t(std::atoll(f + n + 1)));
 }
 
 nrsense_status dev_alloc(nrsense_plan_s* p, void** ptr, size_t bytes) {
   *ptr = nullptr;
   if (bytes == 0) return NRSENSE_OK;
-  if (fault_requested("alloc")) return NRSENSE_ERR_OOM;
+  if (fault_requested("alloc", p)) return NRSENSE_ERR_OOM;
   if (cudaMalloc(ptr, bytes) != cudaSuccess) {
     cudaGetLastError();
     *ptr = nullptr;
@@ -60,6 +65,20 @@ void dev_free(nrsense_plan_s* p, void* ptr) {
       return;
     }
 }
+
+// Frees what the plan allocated since its construction unless kept: the arrays of
+// a point order are the plan's only once all of them are there.
+struct Rollback {
+  nrsense_plan_s* p;
+  size_t mark;
+  bool keep = false;
+  explicit Rollback(nrsense_plan_s* plan) : p(plan), mark(plan->allocations.size()) {}
+  Rollback(const Rollback&) = delete;
+  Rollback& operator=(const Rollback&) = delete;
+  ~Rollback() {
+    while (!keep && p->allocations.size() > mark) dev_free(p, p->allocations.back());
+  }
+};
 
 void free_pointset(nrsense_plan_s* p, PointSet* ps) {
   void* arrs[] = {ps->qs, ps->perm, ps->list, ps->items, ps->bins, ps->reduces, ps->iitems,
@@ -554,7 +573,8 @@ nrsense_status sorted_image_points(nrsense_plan_s* p, int shift, bool cells, con
 nrsense_status build_home_set(nrsense_plan_s* p, cudaStream_t s) {
   const Geo& g = p->geo;
   if (p->home_scratch != nullptr) return NRSENSE_OK;  // built
-  HomeSet& hs = p->ihome;
+  Rollback undo(p);
+  HomeSet hs{};
   hs.nt0 = (g.g0 + 7) / 8;
   hs.nt1 = (g.g1 + 7) / 8;
   hs.nt2 = (g.g2 + 7) / 8;
@@ -587,7 +607,12 @@ nrsense_status build_home_set(nrsense_plan_s* p, cudaStream_t s) {
     *cov[a] = dtab;
   }
   if (configure_home_kernels() != cudaSuccess) return NRSENSE_ERR_CUDA;
-  return dev_alloc_n(p, &p->home_scratch, home_scratch_elems(hs));
+  nrsense_c64* scratch = nullptr;
+  NRS_TRY(dev_alloc_n(p, &scratch, home_scratch_elems(hs)));
+  undo.keep = true;
+  p->ihome = hs;
+  p->home_scratch = scratch;
+  return NRSENSE_OK;
 }
 
 // Image-space points sorted by the 4^3 block of their first tap (stable), with
@@ -603,15 +628,14 @@ nrsense_status build_row_set(nrsense_plan_s* p, cudaStream_t s) {
   return NRSENSE_OK;
 }
 
-// scratch for split tiles: slots x coil chunks x tile x chunk coils (grown,
-// never shrunk)
+// scratch for split tiles of the k-space spread: slots x coil chunks x tile x
+// chunk coils (grown, never shrunk)
 nrsense_status ensure_scratch(nrsense_plan_s* p) {
   long long need = 0;
   auto tile_pts = [](const PointSet& ps) {
     return (long long)ps.tp.t0 * ps.tp.t1 * ps.tp.t2;
   };
-  if (!p->identity_warp) need = std::max(need, (long long)p->ipts.n_slots * tile_pts(p->ipts));
-  if (p->C > 0 && !p->kpts.empty()) {
+  if (p->C > 0) {
     const int cc = spread_coil_chunk(p->C);
     const int chunks = (p->C + cc - 1) / cc;
     for (int j0 = 0; j0 < p->P; j0 += p->phase_chunk) {
@@ -631,12 +655,19 @@ nrsense_status ensure_scratch(nrsense_plan_s* p) {
 
 // halo lists of the displaced voxels (the spread over per-tile lists)
 nrsense_status build_image_lists(nrsense_plan_s* p, cudaStream_t s) {
-  if (p->ipts.qs != nullptr) return NRSENSE_OK;
+  if (p->ipts.qs != nullptr) return NRSENSE_OK;  // built
+  Rollback undo(p);
   std::vector<HostPoint> pts;
   NRS_TRY(host_image_points(p, pts, s));
-  NRS_TRY(build_pointset(p, pts, &p->ipts, p->itiles, nullptr, /*interp=*/false, kSpreadMaxItemImage,
-                         s));
-  return ensure_scratch(p);
+  PointSet lists;
+  NRS_TRY(build_pointset(p, pts, &lists, p->itiles, nullptr, /*interp=*/false, kSpreadMaxItemImage, s));
+  // partial tiles of their own: the k-space spread's scratch stays where it is
+  nrsense_c64* scratch = nullptr;
+  NRS_TRY(dev_alloc_n(p, &scratch, (long long)lists.n_slots * lists.tp.t0 * lists.tp.t1 * lists.tp.t2));
+  undo.keep = true;
+  p->ipts = lists;
+  p->image_scratch = scratch;
+  return NRSENSE_OK;
 }
 
 nrsense_status cufft_check(cufftResult r) {

@@ -109,6 +109,7 @@ struct nrsense_plan_s {
   // 0.309 at 128^3 with four, 0.0067 against 0.0148 at 32^3)
   bool interp_home = false;
   nrsense_c64* home_scratch = nullptr;  // super-tile rims of the home-tile spread
+  nrsense_c64* image_scratch = nullptr;  // partial tiles of ipts' split items
   nrs::TilePlan ktiles{}, itiles{};  // k-space and image-space tiles
   int phase_chunk = 1;              // phases per launch
 
@@ -138,7 +139,7 @@ struct nrsense_plan_s {
   bool comp_spread = false;   // desc.precision == NRSENSE_FP32_COMPENSATED
   nrsense_c64* b_y = nullptr;      // Mtot * C
   nrsense_c64* b_tmp = nullptr;    // N^3 (normal operator scratch)
-  nrsense_c64* b_scratch = nullptr;  // partial tiles
+  nrsense_c64* b_scratch = nullptr;  // partial tiles of the k-space spread
   long long scratch_elems = 0;
   int32_t* d_status = nullptr;
 
