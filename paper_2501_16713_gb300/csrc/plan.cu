@@ -645,11 +645,12 @@ nrsense_status ensure_scratch(nrsense_plan_s* p) {
     }
   }
   if (need <= p->scratch_elems) return NRSENSE_OK;
+  nrsense_c64* larger = nullptr;
+  NRS_TRY(dev_alloc_n(p, &larger, need));
   dev_free(p, p->b_scratch);
-  p->b_scratch = nullptr;
-  p->scratch_elems = 0;
-  NRS_TRY(dev_alloc_n(p, &p->b_scratch, need));
+  p->b_scratch = larger;
   p->scratch_elems = need;
+  p->epoch += 1;  // captured graphs hold the old address
   return NRSENSE_OK;
 }
 
@@ -1063,7 +1064,7 @@ nrsense_status ensure_image_sets(nrsense_plan_s* p, bool lists, bool home, cudaS
   return NRSENSE_OK;
 }
 
-nrsense_status retile_kspace(nrsense_plan_s* p, int max_item, cudaStream_t s) {
+static nrsense_status retile_impl(nrsense_plan_s* p, int max_item, cudaStream_t s) {
   p->epoch += 1;  // point-set buffers are rebuilt
   if (max_item < 64 || max_item > (1 << 16)) return NRSENSE_ERR_ARG;
   if (p->C == 0 || max_item == p->spread_max_item) {
@@ -1094,14 +1095,30 @@ nrsense_status retile_kspace(nrsense_plan_s* p, int max_item, cudaStream_t s) {
       pts[i].f[2] = qs[i].z;
       pts[i].row = perm[i];
     }
+    // the phase's new items replace the old ones once they and the scratch that they
+    // need are there: a refused allocation leaves every phase with items that fit
     PointSet fresh;
-    NRS_TRY(build_pointset(p, pts, &fresh, ps.tp, &p->kunion, /*interp=*/true, max_item, s));
-    free_pointset(p, &ps);
-    ps = fresh;
+    {
+      Rollback undo(p);
+      NRS_TRY(build_pointset(p, pts, &fresh, ps.tp, &p->kunion, /*interp=*/true, max_item, s));
+      undo.keep = true;
+    }
+    std::swap(ps, fresh);
+    const nrsense_status st = ensure_scratch(p);
+    if (st != NRSENSE_OK) std::swap(ps, fresh);
+    free_pointset(p, &fresh);
+    if (st != NRSENSE_OK) return st;
   }
   p->spread_max_item = max_item;
-  NRS_TRY(ensure_scratch(p));
   return cudaStreamSynchronize(s) == cudaSuccess ? NRSENSE_OK : NRSENSE_ERR_CUDA;
+}
+
+nrsense_status retile_kspace(nrsense_plan_s* p, int max_item, cudaStream_t s) {
+  try {
+    return retile_impl(p, max_item, s);
+  } catch (const std::bad_alloc&) {
+    return NRSENSE_ERR_OOM;
+  }
 }
 
 }  // namespace nrs

@@ -81,3 +81,30 @@ def test_refused_point_order_is_built_by_the_next_call(monkeypatch, phases, choi
     assert plan.device_status() == 0
     plan.close()
 
+
+def test_refused_work_item_split_leaves_a_plan_that_runs(monkeypatch):
+    """Three phases re-split one after the other, stopped at every allocation: the adjoint
+    and a captured CG solve stay right in between.  Phases already re-split sum their tiles
+    in another order, so results agree to rounding, which three iterations on a system of
+    condition 2 or so carry on without growth."""
+    plan, y, x0, ref = _setup(3, samples=40000)
+    lam = 1e6
+    cg = lambda: plan.solve_cg(y, lam, tol=0.0, maxit=3, graph=True)[0].cpu().numpy()  # noqa: E731
+    cg0 = cg()
+    split = plan.info()["split_tiles"]
+    refused = 0
+    for n in range(1, 300):
+        monkeypatch.setenv("NRSENSE_FAULT", "alloc:%d" % n)
+        st = _set(plan, spread_max_item=512)
+        monkeypatch.delenv("NRSENSE_FAULT")
+        if st == 0:
+            break
+        assert st == -2
+        refused += 1
+        assert rel_l2(plan.adjoint(y).cpu().numpy(), ref) < TOL_FP32
+        assert rel_l2(cg(), cg0) < TOL_FP32
+    assert st == 0 and refused > 5
+    assert plan.info()["split_tiles"] > split
+    assert rel_l2(plan.adjoint(y).cpu().numpy(), ref) < TOL_FP32
+    assert rel_l2(cg(), cg0) < TOL_FP32
+    plan.close()
