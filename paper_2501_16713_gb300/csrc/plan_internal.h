@@ -104,9 +104,8 @@ struct nrsense_plan_s {
   bool rows_ok = false;             // irows built (grids of a multiple of 4, plain FP32)
   bool rows_sparse = false;         // rows_ok, W = 4 and few enough points for the row spread
   bool home_ok = false;             // ihome applies (W = 4, not compensated); built when used
-  // image-space interpolation over super-tiles (autotuned; a thread per voxel
-  // until then: 0.324 against 0.414 ms at 192^3 with one phase, 0.300 against
-  // 0.309 at 128^3 with four, 0.0067 against 0.0148 at 32^3)
+  // image-space interpolation over super-tiles, else a thread per voxel (autotuned;
+  // until then by the number of points per grid value, plan.cu)
   bool interp_home = false;
   nrsense_c64* home_scratch = nullptr;  // super-tile rims of the home-tile spread
   nrsense_c64* image_scratch = nullptr;  // partial tiles of ipts' split items

@@ -1,0 +1,76 @@
+"""The kernels an untuned plan takes, against the ones it could take: a default rule
+picks the faster side of its line.
+
+Times are the library's own stage times, medians over several runs; the sides measured
+here differ by 1.2 and more, the default may lose a tenth.
+"""
+
+import ctypes
+
+import numpy as np
+import pytest
+
+from helpers import crandn, to_dev
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import __graft_entry__ as g
+    g.build()
+
+
+def _contraction(shape, phases, factor):
+    n = np.stack(np.meshgrid(*[np.arange(s, dtype=np.float32) for s in shape], indexing="ij"))
+    c = np.array([(s - 1) / 2 for s in shape], np.float32)[:, None, None, None]
+    return np.stack([(factor - 1.0) * (n - c) + 0.1 * (j + 1) for j in range(phases)]).astype(np.float32)
+
+
+def _stage(plan, name, run, repeat=7):
+    """Median time of a stage, ms."""
+    import torch
+    for _ in range(3):
+        run()
+    ts = []
+    for _ in range(repeat):
+        plan.profile_start(200)
+        for _ in range(4):
+            run()
+        torch.cuda.synchronize()
+        ts.append(plan.profile_stop()[0][name][0] / 4)
+    return sorted(ts)[repeat // 2]
+
+
+def _set(plan, **kw):
+    from paper_2501_16713_gb300.nrsense import Tuning
+    t = Tuning()
+    t.spread_variant, t.interp_coils, t.interp_tma, t.spread_image_warp = 1, 8, 0, 2
+    for k, v in kw.items():
+        setattr(t, k, v)
+    assert plan.lib.nrsense_plan_set_tuning(plan._h, ctypes.byref(t)) == 0
+
+
+@pytest.mark.parametrize("shape,osf,phases", [((64, 64, 64), 1.5, 1), ((128, 128, 128), 1.5, 1),
+                                              ((96, 80, 104), 1.25, 2), ((128, 128, 128), 2, 8),
+                                              ((64, 64, 64), 2.5, 1), ((32, 32, 32), 2, 8),
+                                              ((96, 96, 96), 2, 1)])
+def test_image_interpolation(shape, osf, phases):
+    import torch
+    from paper_2501_16713_gb300 import Plan
+    plan = Plan(shape, disp=to_dev(_contraction(shape, phases, 0.95)), n_phases=phases, osf=osf)
+    x = to_dev(crandn(np.random.default_rng(161), shape))
+    out = plan.warp_forward(x)
+    run = lambda: plan.warp_forward(x, out=out)  # noqa: E731
+    ms, first = _stage(plan, "interp_image", run), out.clone()
+    other = []
+    for home in (0, 1):
+        _set(plan, interp_image_home=home)
+        other.append(_stage(plan, "interp_image", run))
+        assert torch.equal(out, first)
+    print(shape, osf, phases, "default %.4f, per voxel %.4f, super-tiles %.4f ms" % (ms, *other))
+    assert ms < 1.1 * min(other)
+    plan.close()
