@@ -616,14 +616,37 @@ nrsense_status build_home_set(nrsense_plan_s* p, cudaStream_t s) {
 }
 
 // Image-space points sorted by the 4^3 block of their first tap (stable), with
-// the first sorted index of every block (spread_rows.cu).
+// the first sorted index of every block (spread_rows.cu); not kept (rows_ok stays
+// false) where the displacement gathers the points in so few rows that the warp with
+// the most of them decides the time: a row is one warp's, about 30 (W = 4) or 48 ns a
+// point, while the home tiles (W = 4) and the split halo lists (W = 6) deal a crowd to
+// more warps.  T^H of images contracted about their centre, points of the fullest warp,
+// rows against home tiles: 64^3 540 0.053 / 0.053 ms, 1280 0.092 / 0.082; 128^3 1656
+// 0.262 / 0.304, 4096 0.361 / 0.296, 15876 0.825 / 0.447.  W = 6 against halo lists: 64^3
+// 3456 0.35 / 0.70, 16000 0.94 / 1.00, 78400 3.7 / 1.05; 128^3 9792 1.21 / 2.64, 34400
+// 3.15 / 2.81, 172800 9.5 / 2.93.  Motion of some voxels stays far below: 160 to 1250 at
+// 16^3 to 192^3.
 nrsense_status build_row_set(nrsense_plan_s* p, cudaStream_t s) {
   const Geo& g = p->geo;
-  RowSet& rs = p->irows;
+  Rollback undo(p);
+  RowSet rs{};
   rs.nb0 = g.g0 / 4;
   rs.nb1 = g.g1 / 4;
   rs.nb2 = g.g2 / 4;
   NRS_TRY(sorted_image_points(p, 2, false, &rs.qs, &rs.perm, &rs.start, s));
+  int32_t* most = nullptr;
+  int32_t load = 0;
+  NRS_TRY(dev_alloc_n(p, &most, 1));
+  if (cudaMemsetAsync(most, 0, sizeof(load), s) != cudaSuccess) return NRSENSE_ERR_CUDA;
+  launch_row_load(p->W, rs, most, s);
+  if (cudaMemcpyAsync(&load, most, sizeof(load), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+      cudaStreamSynchronize(s) != cudaSuccess)
+    return NRSENSE_ERR_CUDA;
+  dev_free(p, most);
+  const long long n = (long long)p->P * g.nvox;
+  if (load > (p->W == 4 ? 400 + n / 1000 : 16000 + n / 128)) return NRSENSE_OK;
+  undo.keep = true;
+  p->irows = rs;
   p->rows_ok = true;
   return NRSENSE_OK;
 }
@@ -805,16 +828,11 @@ nrsense_status create_impl(nrsense_plan_s* p, const nrsense_desc* desc, const in
     // visits per point
     const bool rows = !p->comp_spread && !p->grid_bf16 && g.g0 % 4 == 0 && g.g1 % 4 == 0 &&
                       g.g2 % 4 == 0;
-    p->rows_sparse = rows && p->W == 4 && 6 * p->P * g.nvox <= g.ngrid;
     p->home_ok = p->W == 4 && !p->comp_spread;
     if (p->home_ok) p->spread_image_variant = kSpreadHome;
-    if (rows && (p->W != 4 || p->rows_sparse)) {
-      NRS_TRY(build_row_set(p, s));
-    } else if (p->home_ok) {
-      NRS_TRY(build_home_set(p, s));
-    } else {
-      NRS_TRY(build_image_lists(p, s));
-    }
+    if (rows && (p->W != 4 || 6 * p->P * g.nvox <= g.ngrid)) NRS_TRY(build_row_set(p, s));
+    p->rows_sparse = p->rows_ok && p->W == 4;
+    if (!p->rows_ok) NRS_TRY(p->home_ok ? build_home_set(p, s) : build_image_lists(p, s));
     // Interpolation until the plan is tuned (bitwise the same values): a thread per
     // voxel, or from super-tiles staged in shared memory.  Per voxel at sigma 2: 0.324
     // against 0.429 ms at 192^3 with one phase, 0.302 against 0.311 at 128^3 with four;

@@ -101,7 +101,8 @@ struct nrsense_plan_s {
   nrs::PointSet ipts;               // displaced voxels of all phases
   nrs::HomeSet ihome{};             // the same, sorted by 8^3 home tile (home-tile spread)
   nrs::RowSet irows{};              // the same, sorted by 4^3 block (row spread)
-  bool rows_ok = false;             // irows built (grids of a multiple of 4, plain FP32)
+  bool rows_ok = false;             // irows built (grids of a multiple of 4, plain FP32, the
+                                    // points not crowded into a few rows)
   bool rows_sparse = false;         // rows_ok, W = 4 and few enough points for the row spread
   bool home_ok = false;             // ihome applies (W = 4, not compensated); built when used
   // image-space interpolation over super-tiles, else a thread per voxel (autotuned;
@@ -339,6 +340,9 @@ int launch_spread_home(const Geo& g, const KernelCoefs& kc, const HomeSet& hs,
                        const nrsense_c64* vals, nrsense_c64* grid, nrsense_c64* scratch,
                        cudaStream_t s);
 long long home_scratch_elems(const HomeSet& hs);
+// largest number of points a warp of the row spread visits, into *most (zeroed
+// before; spread_rows.cu)
+int launch_row_load(int W, const RowSet& rs, int32_t* most, cudaStream_t s);
 // row spread on the tensor cores (spread_rows.cu): all points of `rs` into grid
 int launch_spread_rows(const Geo& g, int W, const KernelCoefs& kc, const RowSet& rs,
                        const nrsense_c64* vals, nrsense_c64* grid, cudaStream_t s);

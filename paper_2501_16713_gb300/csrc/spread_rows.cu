@@ -240,6 +240,30 @@ int row_segment(const RowSet& rs) {
   return int(std::min<long long>(seg, rs.nb2));
 }
 
+// Points that a warp of launch_spread_rows visits, the largest over its warps.
+__global__ void row_load_kernel(RowSet rs, int K, int seg, int segs, int32_t* __restrict__ most) {
+  const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  if (i >= (long long)rs.nb0 * rs.nb1 * segs) return;
+  const int xs = int(i % segs) * seg, xe = min(xs + seg, rs.nb2), lead = xs - (K - 1);
+  const int by = int(i / segs % rs.nb1), bz = int(i / segs / rs.nb1);
+  int load = 0;
+  for (int d = 0; d < K; ++d)
+    for (int e = 0; e < K; ++e) {
+      const int pz = bz >= d ? bz - d : bz - d + rs.nb0, py = by >= e ? by - e : by - e + rs.nb1;
+      const int32_t* st = rs.start + ((long long)pz * rs.nb1 + py) * rs.nb2;
+      load += st[xe] - st[max(lead, 0)];
+      if (lead < 0) load += st[rs.nb2] - st[rs.nb2 + lead];
+    }
+  atomicMax(most, load);
+}
+
+int launch_row_load(int W, const RowSet& rs, int32_t* most, cudaStream_t s) {
+  const int seg = row_segment(rs), segs = (rs.nb2 + seg - 1) / seg;
+  const long long n = (long long)rs.nb0 * rs.nb1 * segs;
+  row_load_kernel<<<unsigned((n + 255) / 256), 256, 0, s>>>(rs, W == 4 ? 2 : 3, seg, segs, most);
+  return 1;
+}
+
 int launch_spread_rows(const Geo& g, int W, const KernelCoefs& kc, const RowSet& rs,
                        const nrsense_c64* vals, nrsense_c64* grid, cudaStream_t s) {
   const int seg = row_segment(rs);

@@ -74,3 +74,28 @@ def test_image_interpolation(shape, osf, phases):
     print(shape, osf, phases, "default %.4f, per voxel %.4f, super-tiles %.4f ms" % (ms, *other))
     assert ms < 1.1 * min(other)
     plan.close()
+
+
+@pytest.mark.parametrize("width,factor,rows", [(4, 1.0, True), (4, 0.8, True), (4, 0.5, False),
+                                               (4, 0.15, False), (6, 1.0, True), (6, 0.5, True),
+                                               (6, 0.15, False), (6, 0.05, False)])
+def test_image_spread_of_crowded_points(width, factor, rows):
+    """Images contracted about their centre: block rows (one kernel) until the crowd is one
+    warp's, then home tiles or split halo lists (two)."""
+    import torch
+    from paper_2501_16713_gb300 import Plan
+    shape = (128, 128, 128)
+    w = to_dev(crandn(np.random.default_rng(162), (1,) + shape))
+
+    def kernels(factor):
+        plan = Plan(shape, disp=to_dev(_contraction(shape, 1, factor)), n_phases=1, width=width)
+        out = plan.warp_adjoint(w)
+        plan.profile_start(100)
+        plan.warp_adjoint(w, out=out)
+        torch.cuda.synchronize()
+        st, own = plan.profile_stop()
+        print(width, factor, "%.4f ms, %d kernels" % (st["spread_image"][0], own))
+        plan.close()
+        return own
+
+    assert kernels(factor) - kernels(1.0) == (0 if rows else 1)
