@@ -73,7 +73,7 @@ struct PhaseTable {
   const int32_t* perm[kMaxChunkPhases];
   const int2* list[kMaxChunkPhases];
   const int32_t* bins[kMaxChunkPhases];
-  const int2* clist[kMaxChunkPhases];     // class-ordered lists (8^3 tiles, W = 4), or null
+  const int2* clist[kMaxChunkPhases];     // class-ordered lists (8^3 tiles), or null
   const int32_t* cbins[kMaxChunkPhases];  // kCubeBins class starts per item
   const SpreadItem* items[kMaxChunkPhases];
   const ReduceItem* reduces[kMaxChunkPhases];
@@ -82,6 +82,7 @@ struct PhaseTable {
   int red0[kMaxChunkPhases + 1];      // prefix sums of reduce items per phase
   int slot0[kMaxChunkPhases];         // first scratch slot of the phase
   int nphase;
+  long long entries;                  // k-space spread: list entries of all items
 };
 
 // Image-space points (the displaced voxels of all phases) sorted by the 8^3

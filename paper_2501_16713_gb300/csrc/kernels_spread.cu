@@ -1283,6 +1283,27 @@ void launch_few(const Geo& g, const KernelCoefs& kc, int C, const TilePlan& tp, 
       g, kc, C, tp, pt, vals, grids, scratch);
 }
 
+// Whether the sub-block kernel of one to four coils pays on an untuned plan.  It spends
+// a warp on every sub-block of an item and stores 16 bytes a lane, so it loses where
+// items hold a few points only and their tiles outgrow the L2 cache; the kernels with a
+// CTA per tile lose by their barriers, once items hold more.  Cone trajectories at
+// sigma 2, ms (e: entries per item):
+//   2 coils, W = 4 (register kernel): 40 k samples at 64^3 (e 45) 0.101 -> 0.070, 3 M at
+//   128^3 (e 354) 1.14 -> 0.78, 20 k at 128^3 (e 8, 56 MB of tiles) 0.089 -> 0.080; but 100 k
+//   at 128^3 (e 15, 142 MB) 0.187 -> 0.200, at 192^3 (e 6, 353 MB) 0.293 -> 0.370, 10 k at
+//   256^3 (e 4, 58 MB) 0.051 -> 0.060.
+//   1 coil, and W = 6 (generic kernel): 100 k at 128^3 0.305 -> 0.179 (W = 6, 1 coil), 0.540
+//   -> 0.438 (3 coils, 223 MB); but 200 k at 256^3 (e 5 to 7) 0.500 -> 0.559 (W = 4, 1 coil, 441
+//   MB), 0.673 -> 0.769 (W = 6), 0.85 -> 1.18 (2 coils), 1.24 -> 2.13 (3 coils, e 7), and with 3
+//   coils 40 k at 192^3 (e 6, 351 MB) 0.39 -> 0.48, 10 k at 256^3 (e 4, 123 MB) 0.130 -> 0.161.
+bool few_pays(const PhaseTable& pt, int W, int C) {
+  const double items = pt.item0[pt.nphase], e = pt.entries / std::max(items, 1.0);
+  const double tiles_mb = items * 512 * sizeof(float2) * C * 1e-6;
+  if (e >= 32.0) return true;
+  if (W == 4 && C > 1) return e >= 6.5 && tiles_mb <= 85.0;
+  return tiles_mb <= 250.0 && (C <= 2 || e >= 5.5);
+}
+
 template <int CC, typename GT, bool COMP>
 int dispatch_coils(const Geo& g, const KernelCoefs& kc, int C, const TilePlan& tp,
                    const PhaseTable& pt, const float2* vals, GT* grids, float2* scratch,
@@ -1297,8 +1318,8 @@ int dispatch_coils(const Geo& g, const KernelCoefs& kc, int C, const TilePlan& t
     const size_t smem = size_t(8 * 8 * 8) * CC * sizeof(float2) * (COMP ? 2 : 1);
     spread_coils_kernel<CC, GT, COMP><<<grid, kThreads, smem, s>>>(g, kc, C, tp, pt, vals, grids,
                                                                    scratch);
-  } else if (CC < 8 && sizeof(GT) == 8 && (variant == kSpreadMMA || variant == kSpreadCubeExact) &&
-             pt.clist[0] != nullptr) {
+  } else if (CC < 8 && sizeof(GT) == 8 && pt.clist[0] != nullptr &&
+             (variant == kSpreadMMA || (variant == kSpreadCubeExact && few_pays(pt, 4, C)))) {
     if constexpr (CC < 8 && sizeof(GT) == 8) launch_few<CC, 4>(g, kc, C, tp, pt, vals, grids, scratch, s);
   } else if (CC == 8 && ((variant == kSpreadMMA && mma_cube) || variant == kSpreadCubeExact) &&
              pt.clist[0] != nullptr) {
@@ -1340,13 +1361,13 @@ template <typename GT, bool COMP>
 int spread_multi(const Geo& g, int W, const KernelCoefs& kc, int C, const TilePlan& tp,
                  const PhaseTable& pt, const float2* v, GT* gr, float2* sc, int variant,
                  cudaStream_t s) {
-  // FP32 grids with class lists (k space): one coil, and W = 6, always take the
-  // sub-block kernels; the alternative is the generic kernel (one coil, 16 k
-  // samples on 128^3: 0.100 -> 0.044 ms; W = 6, 8 coils, 2 x 150 k samples on 144 x
-  // 120 x 96: 1.42 -> 0.33 ms with errors of 7.4e-7 to 9.4e-7 against 64 bits,
-  // the generic kernel's 1.2e-6)
+  // FP32 grids with class lists (k space): one coil, and W = 6, take the sub-block
+  // kernels, with few coils where they pay; the alternative is the generic kernel (one
+  // coil, 16 k samples on 128^3: 0.100 -> 0.044 ms; W = 6, 8 coils, 2 x 150 k samples on
+  // 144 x 120 x 96: 1.42 -> 0.33 ms with errors of 7.4e-7 to 9.4e-7 against 64 bits,
+  // the generic kernel's 1.2e-6; 200 k at 256^3 2.19 -> 1.27)
   if constexpr (sizeof(GT) == 8 && !COMP) {
-    if (pt.clist[0] != nullptr && (C == 1 || W == 6)) {
+    if (pt.clist[0] != nullptr && (C == 1 || W == 6) && (C > 4 || few_pays(pt, W, C))) {
       const int cc = spread_coil_chunk(C), chunks = (C + cc - 1) / cc;
       if (W == 4) {
         launch_few<1, 4>(g, kc, C, tp, pt, v, gr, sc, s);

@@ -1039,9 +1039,10 @@ nrsense_status create_impl(nrsense_plan_s* p, const nrsense_desc* desc, const in
     // sub-blocks with FP32-accurate sums: on the tensor cores, eight points per
     // rounded addition (5 to 8 coils and chunks of 8; 256^3, 16 coils, 3 M
     // samples: below 4.20 ms against 6.50 of the register kernel, the adjoint's error
-    // 2.6e-7 against 2.7e-7), or by FMAs (2 coils at 64^3, 100 k samples: 0.091 against
-    // 0.137 ms; with 3 and 4 coils the register kernel is the faster one on dense
-    // samples, 0.495 against 0.634 ms at 128^3, and the tuner times both).  BF16 grids keep the register kernel and its exact summation order.
+    // 2.6e-7 against 2.7e-7), or by FMAs (1 and 2 coils, where items hold enough points:
+    // few_pays, kernels_spread.cu; with 3 and 4 coils the register kernel is the faster
+    // one on dense samples, 0.495 against 0.634 ms at 128^3, and the tuner times both).
+    // BF16 grids keep the register kernel and its exact summation order.
     if (p->tma_ok) {
       p->interp_tma = true;
       p->interp_coils = p->C <= 2 ? 2 : 4;

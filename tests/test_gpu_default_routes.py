@@ -10,7 +10,9 @@ import ctypes
 import numpy as np
 import pytest
 
-from helpers import crandn, to_dev
+import synth
+from helpers import TOL_FP32, crandn, make_plan, rel_l2, to_dev
+from oracle import operators as O
 
 pytestmark = pytest.mark.gpu
 
@@ -99,3 +101,38 @@ def test_image_spread_of_crowded_points(width, factor, rows):
         return own
 
     assert kernels(factor) - kernels(1.0) == (0 if rows else 1)
+
+
+@pytest.mark.parametrize("n,samples", [(64, 40000), (128, 20000), (192, 100000), (64, 2000000)])
+def test_two_coil_spread(n, samples):
+    """The sub-block kernel only where items hold enough points: against it and the register
+    kernel."""
+    import torch
+    from paper_2501_16713_gb300 import Plan
+    gen = torch.Generator(device="cuda").manual_seed(163)
+    k = (torch.rand((samples, 3), device="cuda", generator=gen) * 2 - 1) * 3.1
+    maps = torch.ones((2, n, n, n), dtype=torch.complex64, device="cuda")
+    plan = Plan((n, n, n), coords=[k], smaps=maps, identity_warp=True)
+    y = torch.randn((samples, 2), dtype=torch.complex64, device="cuda", generator=gen)
+    out = plan.adjoint(y)
+    run = lambda: plan.adjoint(y, out=out)  # noqa: E731
+    ms, other = _stage(plan, "spread_kspace", run), []
+    for variant in (1, 4):
+        _set(plan, spread_variant=variant)
+        other.append(_stage(plan, "spread_kspace", run))
+    print(n, samples, "default %.4f, register %.4f, sub-blocks %.4f ms" % (ms, *other))
+    assert ms < 1.1 * min(other)
+    plan.close()
+
+
+@pytest.mark.parametrize("shape,width,coils,samples", [
+    ((24, 20, 28), 4, 2, 120), ((24, 20, 28), 4, 2, 900), ((24, 20, 28), 6, 3, 60),
+    ((24, 20, 28), 6, 4, 60), ((24, 20, 28), 6, 3, 900), ((18, 22, 20), 6, 3, 30)])
+def test_few_coils_on_both_sides_of_the_line(shape, width, coils, samples):
+    c = synth.small_case(shape, coils, 2, [samples, samples // 2], seed=164, uniform_coords=True)
+    plan = make_plan(c, shape, identity_warp=True, width=width)
+    y = crandn(np.random.default_rng(165), (samples + samples // 2, coils))
+    ref = O.stacked_adjoint(O.Geometry(shape, width=width), np.split(y.astype(np.complex128), [samples]),
+                            [None, None], c["smaps"], c["coords"])
+    assert rel_l2(plan.adjoint(to_dev(y)).cpu().numpy(), ref) < TOL_FP32
+    plan.close()
