@@ -1024,7 +1024,15 @@ nrsense_status create_impl(nrsense_plan_s* p, const nrsense_desc* desc, const in
     // points (64^3, 8 coils, 2 phases: 0.256 against 0.294 ms per E), the
     // power-of-two ones with 256 (128^3, 4 phases: 3.16 against 3.45) and,
     // barely, with 32 and 64
-    p->coil_mixed = p->mix[0].N > 0 && (!p->fft_pruned_ok || std::max(g.g0, std::max(g.g1, g.g2)) == 128);
+    // Grids of 1024 points along z and about as many along another axis stay with
+    // cuFFT: at 1024 points, its best length, the in-place passes hold 131 KB of shared
+    // memory, a CTA per SM, and transform the zero half too.  Two coils forward and
+    // adjoint, own passes against cuFFT: 1024^3 40.9 / 31.8 ms (24.6 / 22.5 at sigma 4),
+    // 1024 x 192 x 960 13.3 / 11.9, 1024 x 1024 x 64 (four coils) 4.6 / 3.9; but 1024 x 864 x
+    // 864 25.1 / 31.1, 512 x 1024 x 1024 14.8 / 18.9, 960^3 34.4 / 47.1.
+    const bool cufft_1024 = g.g0 == 1024 && (g.g1 == 1024 || g.g2 >= 896);
+    p->coil_mixed = p->mix[0].N > 0 && !cufft_1024 &&
+                    (!p->fft_pruned_ok || std::max(g.g0, std::max(g.g1, g.g2)) == 128);
     // tensor maps of the interpolation input (TMA-staged halos, W = 4)
     const long long slots = (long long)p->C * p->phase_chunk;
     // a test-only limit on the halo wait (0 makes every TMA-staged CTA time out)

@@ -136,3 +136,29 @@ def test_few_coils_on_both_sides_of_the_line(shape, width, coils, samples):
                             [None, None], c["smaps"], c["coords"])
     assert rel_l2(plan.adjoint(to_dev(y)).cpu().numpy(), ref) < TOL_FP32
     plan.close()
+
+
+@pytest.mark.parametrize("shape,osf,own", [((256, 256, 12), 4, False), ((256, 32, 224), 4, False),
+                                           ((256, 32, 32), 4, True), ((32, 256, 224), 4, True)])
+def test_coil_transforms_at_1024_points(shape, osf, own):
+    """cuFFT along z of 1024 points and another long axis, own passes else; either way the
+    adjoint of the forward operator (whose parts are held against the oracle at small sizes)."""
+    import torch
+    from paper_2501_16713_gb300 import Plan
+    gen = torch.Generator(device="cuda").manual_seed(166)
+    k = (torch.rand((5000, 3), device="cuda", generator=gen) * 2 - 1) * 3.1
+    maps = torch.randn((1,) + shape, dtype=torch.complex64, device="cuda", generator=gen)
+    plan = Plan(shape, coords=[k], smaps=maps, identity_warp=True, osf=osf)
+    x = torch.randn(shape, dtype=torch.complex64, device="cuda", generator=gen)
+    y = torch.randn((5000, 1), dtype=torch.complex64, device="cuda", generator=gen)
+    plan.forward(x)
+    plan.profile_start(100)
+    ax, ahy = plan.forward(x), plan.adjoint(y)
+    torch.cuda.synchronize()
+    st = plan.profile_stop()[0]
+    assert (st["fft_pruned"][1] > 0, st["fft_gc"][1] > 0) == (own, not own)
+    a = (ax.conj().to(torch.complex128) * y).sum()
+    b = (x.conj().to(torch.complex128) * ahy).sum()
+    scale = ax.to(torch.complex128).norm() * y.to(torch.complex128).norm()
+    assert abs(a - b) < 1e-6 * scale
+    plan.close()
