@@ -452,6 +452,9 @@ nrsense_status build_pointset(nrsense_plan_s* p, const std::vector<HostPoint>& p
   return upload_pointset(p, hs, ps, s);
 }
 
+// samples whose host lists a plan's creation holds at once (several phases)
+constexpr long long kHostListPoints = 8 << 20;
+
 // f(j) for j < n in threads (at most one per core); the first failure's status.
 template <class F>
 nrsense_status for_phases(int n, F&& f) {
@@ -925,16 +928,25 @@ nrsense_status create_impl(nrsense_plan_s* p, const nrsense_desc* desc, const in
       NRS_TRY(dev_alloc_n(p, &p->kanymask, (long long)am.size()));
       NRS_TRY(upload(p->kanymask, am, s));
     }
-    std::vector<HostSet> sets((size_t)p->P);
-    NRS_TRY(for_phases(p->P, [&](int j) -> nrsense_status {
-      const nrsense_status st = compute_pointset(g, p->W, all[(size_t)j], ktiles, &uni, /*interp=*/true,
-                                                 p->spread_max_item, &sets[(size_t)j]);
-      std::vector<HostPoint>().swap(all[(size_t)j]);
-      return st;
-    }));
-    for (int j = 0; j < p->P; ++j) {
-      NRS_TRY(upload_pointset(p, sets[(size_t)j], &p->kpts[j], s));
-      sets[(size_t)j] = HostSet{};
+    // The phases' lists in turn, as many at once as hold kHostListPoints samples
+    // together: about 120 bytes of host memory a sample, 1 GB, beside the samples' own
+    // records (one phase alone takes what it needs).
+    for (int j0 = 0; j0 < p->P;) {
+      int j1 = j0;
+      for (long long n = 0; j1 < p->P && (j1 == j0 || n + p->M[j1] <= kHostListPoints); ++j1) n += p->M[j1];
+      std::vector<HostSet> sets((size_t)(j1 - j0));
+      NRS_TRY(for_phases(j1 - j0, [&](int k) -> nrsense_status {
+        std::vector<HostPoint>& pts = all[(size_t)(j0 + k)];
+        const nrsense_status st = compute_pointset(g, p->W, pts, ktiles, &uni, /*interp=*/true,
+                                                   p->spread_max_item, &sets[(size_t)k]);
+        std::vector<HostPoint>().swap(pts);
+        return st;
+      }));
+      for (; j0 < j1; ++j0) {
+        HostSet& hs = sets[sets.size() - size_t(j1 - j0)];
+        NRS_TRY(upload_pointset(p, hs, &p->kpts[(size_t)j0], s));
+        hs = HostSet{};
+      }
     }
     p->kunion.swap(uni);
   }
