@@ -50,7 +50,7 @@ def _stage(plan, name, run, repeat=7):
 def _set(plan, **kw):
     from paper_2501_16713_gb300.nrsense import Tuning
     t = Tuning()
-    t.spread_variant, t.interp_coils, t.interp_tma, t.spread_image_warp = 1, 8, 0, 2
+    t.spread_variant, t.interp_coils, t.interp_tma, t.spread_image_warp = 1, 8, 0, 0
     for k, v in kw.items():
         setattr(t, k, v)
     assert plan.lib.nrsense_plan_set_tuning(plan._h, ctypes.byref(t)) == 0
@@ -69,8 +69,9 @@ def test_image_interpolation(shape, osf, phases):
     run = lambda: plan.warp_forward(x, out=out)  # noqa: E731
     ms, first = _stage(plan, "interp_image", run), out.clone()
     other = []
+    own = int(osf == 2 and set(shape) <= {16, 32, 64, 128})  # power-of-two transforms, as created
     for home in (0, 1):
-        _set(plan, interp_image_home=home)
+        _set(plan, interp_image_home=home, spread_image_warp=2, image_fft_pruned=own)
         other.append(_stage(plan, "interp_image", run))
         assert torch.equal(out, first)
     print(shape, osf, phases, "default %.4f, per voxel %.4f, super-tiles %.4f ms" % (ms, *other))
