@@ -11,14 +11,16 @@ namespace nrs {
 
 // Coefficients of the per-tap kernel polynomials (see kb_host.cu):
 // weight of tap t for fractional offset f in [0, 1) is
-//   c(f + W/2 - 1 - t) ~= sum_k coef[k][t] * s^k,  s = 2f - 1.
-// The taps of one power are neighbours, so that two taps' coefficients load and
-// multiply as a pair.
+//   c(f + W/2 - 1 - t) ~= sum_k c[k][t] * s^k,  s = 2f - 1.
+// c: the taps of one power are neighbours, so that two taps' coefficients load and
+// multiply as a pair; t: the powers of one tap, for the kernels that the compiler
+// schedules better that way (kernel_weights_by_tap).
 constexpr int kNumCoef = 10;
 constexpr int kMaxWidth = 6;
 
 struct alignas(8) KernelCoefs {
   float c[kNumCoef][kMaxWidth];
+  float t[kMaxWidth][kNumCoef];
 };
 
 // Per-axis geometry passed by value to every kernel.
@@ -171,6 +173,22 @@ __device__ __forceinline__ void kernel_weights(float f, const KernelCoefs& kc, f
     float acc = kc.c[kNumCoef - 1][t];
 #pragma unroll
     for (int k = kNumCoef - 2; k >= 0; --k) acc = fmaf(acc, s, kc.c[k][t]);
+    w[t] = acc;
+  }
+}
+
+// The same from the tap-major coefficients (bitwise: the same operations).  Spread of
+// the compensated plans with four coils 0.124 against 0.140 ms (32^3, 40 k samples), with two
+// 0.152 against 0.148; per-voxel image interpolation at 128^3, W = 4, 0.096 against 0.101 ms
+// of the paired weights, W = 6 0.246 against 0.232.
+template <int W>
+__device__ __forceinline__ void kernel_weights_by_tap(float f, const KernelCoefs& kc, float (&w)[W]) {
+  const float s = fmaf(2.0f, f, -1.0f);
+#pragma unroll
+  for (int t = 0; t < W; ++t) {
+    float acc = kc.t[t][kNumCoef - 1];
+#pragma unroll
+    for (int k = kNumCoef - 2; k >= 0; --k) acc = fmaf(acc, s, kc.t[t][k]);
     w[t] = acc;
   }
 }

@@ -104,7 +104,7 @@ double fit_kernel_polys(int width, double beta, KernelCoefs* out) {
       b[i] = kb_kernel(f + 0.5 * width - 1.0 - t, width, beta);
     }
     solve_dense(V, b, n);
-    for (int k = 0; k < n; ++k) out->c[k][t] = float(b[k]);
+    for (int k = 0; k < n; ++k) out->c[k][t] = out->t[t][k] = float(b[k]);
     // error of the FP32 Horner evaluation (as on the GPU) against FP64 c
     for (int i = 0; i <= 4000; ++i) {
       const float f = float(i) / 4000.0f;

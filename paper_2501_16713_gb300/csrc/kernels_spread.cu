@@ -222,9 +222,15 @@ __global__ void __launch_bounds__(kThreads) spread_coils_kernel(
         if (r2 < 0) r2 += g.g2;
         if (r2 >= T) r2 -= g.g2;
         float wz[W], wy[W], wx[W];
-        kernel_weights<W>(qq.x, kc, wz);
-        kernel_weights<W>(qq.y, kc, wy);
-        kernel_weights<W>(qq.z, kc, wx);
+        if constexpr (CC == 4) {
+          kernel_weights_by_tap<W>(qq.x, kc, wz);
+          kernel_weights_by_tap<W>(qq.y, kc, wy);
+          kernel_weights_by_tap<W>(qq.z, kc, wx);
+        } else {
+          kernel_weights<W>(qq.x, kc, wz);
+          kernel_weights<W>(qq.y, kc, wy);
+          kernel_weights<W>(qq.z, kc, wx);
+        }
         const int t0 = lz - r0;
         const float wzt = ((unsigned)t0 < (unsigned)W) ? select_tap<W>(wz, t0) : 0.f;
         CoilStage<CC>& d = st[lane];
