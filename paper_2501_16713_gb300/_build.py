@@ -37,6 +37,10 @@ SOURCES = [
     "fft_pruned.cu",
     "fft_mixed.cu",
     "fft_mixed_static.cu",
+    "fft_mixed_static_b.cu",
+    "fft_mixed_static_c.cu",
+    "fft_mixed_static_d.cu",
+    "fft_mixed_static_e.cu",
     "fft_mixed_rt_coil.cu",
     "fft_mixed_rt_image.cu",
     "fft_mixed_gen_coil.cu",

@@ -463,5 +463,18 @@ void run_image_pass(const MixPass& a, const AX& ax, cudaStream_t s) {
   }
 }
 
+// The pass with compile-time radices; false: the axis has other ones.
+template <int R, int S>
+bool pass_for(const MixPass& a, const MixAxis& x, cudaStream_t s) {
+  if (x.R != R || x.S != S) return false;
+  DoubleAxis<StLen<R, S>> ax;
+  ax.l.tw = x.tw_g;
+  if (a.pass < 6)
+    run_coil_pass(a, ax, s);
+  else
+    run_image_pass(a, ax, s);
+  return true;
+}
+
 }  // namespace mixed
 }  // namespace nrs
