@@ -1032,10 +1032,13 @@ nrsense_status create_impl(nrsense_plan_s* p, const nrsense_desc* desc, const in
     // times both paths)
     p->fft_pruned_ok = pruned_fft_supported(g, p->C, p->grid_bf16) && init_pruned_fft() == cudaSuccess;
     p->fft_pruned = p->fft_pruned_ok;
-    // power-of-two grids: the mixed-radix kernels are the faster ones with 128
-    // points (64^3, 8 coils, 2 phases: 0.256 against 0.294 ms per E), the
-    // power-of-two ones with 256 (128^3, 4 phases: 3.16 against 3.45) and,
-    // barely, with 32 and 64
+    // Power-of-two grids up to 256 have both kinds of passes; the mixed-radix ones are the
+    // faster along 128 points, the power-of-two ones along 256 and, barely, along 32 and
+    // 64.  Mixed against power-of-two, ms forward and adjoint, 8 coils, one / four phases: 128^3
+    // grid 0.147 / 0.474 against 0.154 / 0.530, z y x = 128 128 64 0.083 / 0.251 against 0.084 /
+    // 0.275, 128 128 256 0.253 / 0.863 against 0.275 / 0.957; but 64 128 128 0.099 / 0.260 against
+    // 0.087 / 0.266, 128 64 32 0.051 against 0.046, 256^3 0.86 / 3.39 against 0.79 / 3.11.  So by
+    // the two axes whose passes run over the padded columns.
     // Grids of 1024 points along z and about as many along another axis stay with
     // cuFFT: at 1024 points, its best length, the in-place passes hold 131 KB of shared
     // memory, a CTA per SM, and transform the zero half too.  Two coils forward and
@@ -1044,7 +1047,7 @@ nrsense_status create_impl(nrsense_plan_s* p, const nrsense_desc* desc, const in
     // 864 25.1 / 31.1, 512 x 1024 x 1024 14.8 / 18.9, 960^3 34.4 / 47.1.
     const bool cufft_1024 = g.g0 == 1024 && (g.g1 == 1024 || g.g2 >= 896);
     p->coil_mixed = p->mix[0].N > 0 && !cufft_1024 &&
-                    (!p->fft_pruned_ok || std::max(g.g0, std::max(g.g1, g.g2)) == 128);
+                    (!p->fft_pruned_ok || (g.g0 == 128 && g.g1 == 128));
     // tensor maps of the interpolation input (TMA-staged halos, W = 4)
     const long long slots = (long long)p->C * p->phase_chunk;
     // a test-only limit on the halo wait (0 makes every TMA-staged CTA time out)
