@@ -142,7 +142,10 @@ PhaseTable kspace_table(const nrsense_plan_s* p, int j0, int j1, bool spread, lo
     t.row0[jj] = p->off[j0 + jj] - row_base;
     t.item0[jj] = ai;
     ai += spread ? ps.n_items : ps.n_iitems;
-    t.entries += spread ? ps.list_len : 0;
+    if (spread) {
+      t.entries += ps.list_len;
+      t.longest = std::max(t.longest, ps.longest_item);
+    }
     t.red0[jj] = ar;
     ar += spread ? ps.n_reduces : 0;
     t.slot0[jj] = as;

@@ -85,6 +85,7 @@ struct PhaseTable {
   int slot0[kMaxChunkPhases];         // first scratch slot of the phase
   int nphase;
   long long entries;                  // k-space spread: list entries of all items
+  int longest;                        // and of the longest item
 };
 
 // Image-space points (the displaced voxels of all phases) sorted by the 8^3

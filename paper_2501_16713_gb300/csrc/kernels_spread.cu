@@ -1289,25 +1289,34 @@ void launch_few(const Geo& g, const KernelCoefs& kc, int C, const TilePlan& tp, 
       g, kc, C, tp, pt, vals, grids, scratch);
 }
 
-// Whether the sub-block kernel of one to four coils pays on an untuned plan.  It spends
-// a warp on every sub-block of an item and stores 16 bytes a lane, so it loses where
-// items hold a few points only and their tiles outgrow the L2 cache; the kernels with a
-// CTA per tile lose by their barriers, once items hold more.  Cone trajectories at
-// sigma 2, ms (e: entries per item):
-//   2 coils, W = 4 (register kernel): 40 k samples at 64^3 (e 45) 0.101 -> 0.070, 3 M at
-//   128^3 (e 354) 1.14 -> 0.78, 20 k at 128^3 (e 8, 56 MB of tiles) 0.089 -> 0.080; but 100 k
-//   at 128^3 (e 15, 142 MB) 0.187 -> 0.200, at 192^3 (e 6, 353 MB) 0.293 -> 0.370, 10 k at
-//   256^3 (e 4, 58 MB) 0.051 -> 0.060.
-//   1 coil, and W = 6 (generic kernel): 100 k at 128^3 0.305 -> 0.179 (W = 6, 1 coil), 0.540
-//   -> 0.438 (3 coils, 223 MB); but 200 k at 256^3 (e 5 to 7) 0.500 -> 0.559 (W = 4, 1 coil, 441
-//   MB), 0.673 -> 0.769 (W = 6), 0.85 -> 1.18 (2 coils), 1.24 -> 2.13 (3 coils, e 7), and with 3
-//   coils 40 k at 192^3 (e 6, 351 MB) 0.39 -> 0.48, 10 k at 256^3 (e 4, 123 MB) 0.130 -> 0.161.
+// Whether the sub-block kernel of one to four coils is the faster one on a launch's
+// items, by the time that it and its alternative take: so many ns per item (the
+// sub-block kernel spends a warp on each eighth and stores 16 bytes a lane), per list
+// entry, and per entry of the longest item, the serial chain that a CTA per tile works
+// through at a slower rate.  The coefficients are least squares over cone and uniform samples,
+// 500 to 3 M of them on 64^3 to 256^3 at sigma 2, within a tenth or so.  ms, alternative against
+// sub-blocks:
+//   2 coils, W = 4 (register kernel): cones 3 M at 128^3 1.14 / 0.78, 40 k at 64^3 0.101 /
+//   0.070, 100 k at 192^3 0.29 / 0.37, 200 k at 256^3 0.60 / 0.84; uniform 2.5 M at 64^3 0.85 /
+//   0.58, 40 k at 64^3 0.040 / 0.050.
+//   1 coil (generic kernel): cones 100 k at 128^3 0.228 / 0.144, 200 k at 256^3 0.50 / 0.56;
+//   uniform 160 k at 64^3 0.078 / 0.044, 40 k at 128^3 0.099 / 0.164.
+//   W = 6 (generic kernel): cones 100 k at 128^3, 1 coil 0.305 / 0.179, 3 coils 0.54 / 0.44, 200 k
+//   at 256^3, 2 coils 0.85 / 1.18, 3 coils 1.24 / 2.13; uniform 640 k at 128^3, 2 coils 0.90 /
+//   0.53, 10 k 0.093 / 0.195.
 bool few_pays(const PhaseTable& pt, int W, int C) {
-  const double items = pt.item0[pt.nphase], e = pt.entries / std::max(items, 1.0);
-  const double tiles_mb = items * 512 * sizeof(float2) * C * 1e-6;
-  if (e >= 32.0) return true;
-  if (W == 4 && C > 1) return e >= 6.5 && tiles_mb <= 85.0;
-  return tiles_mb <= 250.0 && (C <= 2 || e >= 5.5);
+  struct Ns {
+    double item, entry, longest;
+  };
+  static constexpr Ns kTile[5] = {  // the alternative
+      {2.40, 0.132, 133.0}, {4.33, 0.120, 63.8}, {2.43, 0.224, 174.3}, {2.97, 0.291, 220.6}, {4.38, 0.447, 283.3}};
+  static constexpr Ns kFew[5] = {
+      {4.52, 0.048, 32.2}, {6.93, 0.076, 35.6}, {5.08, 0.070, 34.5}, {7.88, 0.103, 40.3}, {14.5, 0.175, 50.9}};
+  const int k = W == 4 ? std::min(C, 2) - 1 : 1 + std::min(C, 3);
+  auto ns = [&](const Ns& v) {
+    return v.item * pt.item0[pt.nphase] + v.entry * double(pt.entries) + v.longest * pt.longest;
+  };
+  return ns(kFew[k]) < ns(kTile[k]);
 }
 
 template <int CC, typename GT, bool COMP>

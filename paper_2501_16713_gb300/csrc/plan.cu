@@ -194,7 +194,7 @@ void mark_touched_tiles(const nrsense_plan_s* p, const TilePlan& tp,
 struct HostSet {
   TilePlan tp{};
   long long npts = 0, list_len = 0;
-  int occupied = 0, slots = 0;
+  int occupied = 0, slots = 0, longest_item = 0;
   bool cube = false;
   std::vector<float4> qs;
   std::vector<int32_t> perm, bins, cbins;
@@ -348,6 +348,7 @@ nrsense_status compute_pointset(const Geo& g, int W, const std::vector<HostPoint
   });
   hs->slots = slots;
   hs->occupied = occupied;
+  for (const SpreadItem& it : items) hs->longest_item = std::max(hs->longest_item, it.end - it.begin);
   // per item: first entry of each first-tap plane offset bin (list sorted by
   // r0 within every tile, so within every item)
   const int nb = W + tp.t0 + 1;
@@ -425,6 +426,7 @@ nrsense_status upload_pointset(nrsense_plan_s* p, const HostSet& hs, PointSet* p
   ps->n_reduces = int(hs.reds.size());
   ps->n_slots = hs.slots;
   ps->n_occupied = hs.occupied;
+  ps->longest_item = hs.longest_item;
   ps->n_iitems = int(hs.iitems.size());
   auto put = [&](auto** dst, const auto& src) -> nrsense_status {
     NRS_TRY(dev_alloc_n(p, dst, std::max<long long>((long long)src.size(), 1)));
@@ -1062,7 +1064,7 @@ nrsense_status create_impl(nrsense_plan_s* p, const nrsense_desc* desc, const in
     // sub-blocks with FP32-accurate sums: on the tensor cores, eight points per
     // rounded addition (5 to 8 coils and chunks of 8; 256^3, 16 coils, 3 M
     // samples: below 4.20 ms against 6.50 of the register kernel, the adjoint's error
-    // 2.6e-7 against 2.7e-7), or by FMAs (1 and 2 coils, where items hold enough points:
+    // 2.6e-7 against 2.7e-7), or by FMAs (1 and 2 coils, where that is the faster one:
     // few_pays, kernels_spread.cu; with 3 and 4 coils the register kernel is the faster
     // one on dense samples, 0.495 against 0.634 ms at 128^3, and the tuner times both).
     // BF16 grids keep the register kernel and its exact summation order.

@@ -23,6 +23,7 @@ struct TilePlan {
 // voxels of all phases for the image-space adjoint).
 struct PointSet {
   long long npts = 0;
+  int longest_item = 0;         // list entries of the longest spreading item
   TilePlan tp{};                // tiles of this set's spreading/interpolation
   float4* qs = nullptr;         // sorted: (f0, f1, f2, packed base bits)
   int32_t* perm = nullptr;      // sorted index -> value row
