@@ -178,10 +178,12 @@ __device__ __forceinline__ void kernel_weights(float f, const KernelCoefs& kc, f
   }
 }
 
-// The same from the tap-major coefficients (bitwise: the same operations).  Spread of
-// the compensated plans with four coils 0.124 against 0.140 ms (32^3, 40 k samples), with two
-// 0.152 against 0.148; per-voxel image interpolation at 128^3, W = 4, 0.096 against 0.101 ms
-// of the paired weights, W = 6 0.246 against 0.232.
+// The same from the tap-major coefficients (bitwise: the same operations).  Against the
+// paired weights: per-voxel image interpolation at 128^3, W = 4, 0.096 / 0.101 ms, W = 6 0.434 /
+// 0.464 at sigma 1.5 but 0.246 / 0.232 at sigma 2; image interpolation by super-tiles, 128^3,
+// four phases at sigma 1.25, 0.250 / 0.281.  Against the power-major ones of one axis: spread of
+// the compensated plans with four coils 0.124 / 0.140 ms (32^3, 40 k samples), with two 0.152 /
+// 0.148.
 template <int W>
 __device__ __forceinline__ void kernel_weights_by_tap(float f, const KernelCoefs& kc, float (&w)[W]) {
   const float s = fmaf(2.0f, f, -1.0f);

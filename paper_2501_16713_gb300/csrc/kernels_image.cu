@@ -114,7 +114,7 @@ __global__ void __launch_bounds__(256) interp_image_kernel(Geo g, KernelCoefs kc
       b2 = wrap_any(ip2 + int(fl2) - (W / 2 - 1), g.g2);
     }
     float w0[W], w1[W], w2[W];
-    if constexpr (W == 4) {
+    if constexpr (W == 4 || RAT) {
       kernel_weights_by_tap<W>(f0, kc, w0);
       kernel_weights_by_tap<W>(f1, kc, w1);
       kernel_weights_by_tap<W>(f2, kc, w2);

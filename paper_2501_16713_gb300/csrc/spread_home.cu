@@ -331,7 +331,9 @@ __global__ void __launch_bounds__(256) interp_home_kernel(Geo g, KernelCoefs kc,
     int b0, b1, b2;
     unpack_base(__float_as_uint(q.w), b0, b1, b2);
     float w0[4], w1[4], w2[4];
-    kernel_weights3<4>(q.x, q.y, q.z, kc, w0, w1, w2);
+    kernel_weights_by_tap<4>(q.x, kc, w0);
+    kernel_weights_by_tap<4>(q.y, kc, w1);
+    kernel_weights_by_tap<4>(q.z, kc, w2);
     const float2* base = reg + ((b0 - o0) * kHR + (b1 - o1)) * kHR + (b2 - o2);
     float2 aw = make_float2(0.f, 0.f);
 #pragma unroll
