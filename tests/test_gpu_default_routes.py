@@ -163,3 +163,23 @@ def test_coil_transforms_at_1024_points(shape, osf, own):
     scale = ax.to(torch.complex128).norm() * y.to(torch.complex128).norm()
     assert abs(a - b) < 1e-6 * scale
     plan.close()
+
+
+@pytest.mark.parametrize("coils", [2, 3, 4])
+@pytest.mark.parametrize("samples", [50, 40000])
+def test_tuned_sub_blocks_of_few_coils(coils, samples):
+    """The tuner's sub-block choice with two to four coils (partial chunk with three, ragged
+    tiles, split items) against the oracle.  Positive data, FP32 steps of at most some 2.5e-7
+    each: 1e-6 together."""
+    shape = (16, 14, 18)
+    c = synth.small_case(shape, coils, 1, [samples], seed=167)
+    plan = make_plan(c, shape, identity_warp=True)
+    _set(plan, spread_variant=4)
+    y = (1.0 + 0.1 * crandn(np.random.default_rng(168), (samples, coils))).astype(np.complex64)
+    ref = O.stacked_adjoint(O.Geometry(shape), [y.astype(np.complex128)], [None], c["smaps"], c["coords"])
+    yt = to_dev(y)
+    x = plan.adjoint(yt)
+    err = rel_l2(x.cpu().numpy(), ref)
+    print(coils, samples, "adjoint rel L2 %.2e" % err)
+    assert err < 1e-6
+    plan.close()
