@@ -164,37 +164,49 @@ __device__ __forceinline__ void prefetch8(const float2* __restrict__ p, const Vo
   }
 }
 
+// Scale of a Haar pair: orthonormal (the transform entry points), or for the proximal map, whose
+// forward and inverse only meet as a product, sums forward and half sums back: the
+// coefficients of level l come out 2^(1.5 l) times the orthonormal ones and the map
+// back is exact.  The rounded 1/sqrt2, 1.7e-8 short, twice per axis and level would shrink the
+// approximation by 3e-7 in every iteration (three levels), which a FISTA solve adds up
+// to a gain error of 1e-6.
+enum class Scale { kOrthonormal, kSum, kHalfSum };
+
+template <Scale S>
 __device__ __forceinline__ void haar2(float2& a, float2& c) {
-  const float2 s = make_float2((a.x + c.x) * kSqrtHalf, (a.y + c.y) * kSqrtHalf);
-  c = make_float2((a.x - c.x) * kSqrtHalf, (a.y - c.y) * kSqrtHalf);
+  constexpr float k = S == Scale::kOrthonormal ? kSqrtHalf : S == Scale::kSum ? 1.0f : 0.5f;
+  const float2 s = make_float2((a.x + c.x) * k, (a.y + c.y) * k);
+  c = make_float2((a.x - c.x) * k, (a.y - c.y) * k);
   a = s;
 }
 
-// Level 1 inside a group: (a, c) -> ((a + c) / sqrt2, (a - c) / sqrt2) along
-// axes 0, 1, 2; afterwards v[4 s0 + 2 s1 + s2] holds sub-band (s0, s1, s2).
-// The 2 x 2 map is its own inverse, so the inverse runs the axes in reverse.
+// Level 1 inside a group: (a, c) -> k (a + c, a - c) along axes 0, 1, 2; afterwards
+// v[4 s0 + 2 s1 + s2] holds sub-band (s0, s1, s2).  The orthonormal 2 x 2 map is its
+// own inverse, so the inverse runs the axes in reverse.
+template <Scale S>
 __device__ __forceinline__ void haar8_forward(float2 v[8]) {
 #pragma unroll
-  for (int k = 0; k < 4; ++k) haar2(v[k], v[k + 4]);
+  for (int k = 0; k < 4; ++k) haar2<S>(v[k], v[k + 4]);
 #pragma unroll
   for (int k = 0; k < 8; k += 4) {
-    haar2(v[k], v[k + 2]);
-    haar2(v[k + 1], v[k + 3]);
+    haar2<S>(v[k], v[k + 2]);
+    haar2<S>(v[k + 1], v[k + 3]);
   }
 #pragma unroll
-  for (int k = 0; k < 8; k += 2) haar2(v[k], v[k + 1]);
+  for (int k = 0; k < 8; k += 2) haar2<S>(v[k], v[k + 1]);
 }
 
+template <Scale S>
 __device__ __forceinline__ void haar8_inverse(float2 v[8]) {
 #pragma unroll
-  for (int k = 0; k < 8; k += 2) haar2(v[k], v[k + 1]);
+  for (int k = 0; k < 8; k += 2) haar2<S>(v[k], v[k + 1]);
 #pragma unroll
   for (int k = 0; k < 8; k += 4) {
-    haar2(v[k], v[k + 2]);
-    haar2(v[k + 1], v[k + 3]);
+    haar2<S>(v[k], v[k + 2]);
+    haar2<S>(v[k + 1], v[k + 3]);
   }
 #pragma unroll
-  for (int k = 0; k < 4; ++k) haar2(v[k], v[k + 4]);
+  for (int k = 0; k < 4; ++k) haar2<S>(v[k], v[k + 4]);
 }
 
 // Complex soft threshold: c max(0, 1 - tau / |c|), the modulus through the
@@ -208,7 +220,7 @@ __device__ __forceinline__ float2 soft(float2 c, float tau) {
 
 // One lifting pass over the shared array of level-1 approximations (dims
 // g0 x g1 x g2): pairs at distance ST along AXIS.
-template <int J, int ST, int AXIS>
+template <int J, int ST, int AXIS, Scale S>
 __device__ __forceinline__ void haar_pass(float2* s) {
   using D = Box<J>;
   constexpr int d0 = AXIS == 0 ? D::g0 / (2 * ST) : D::g0 / ST;
@@ -225,39 +237,44 @@ __device__ __forceinline__ void haar_pass(float2* s) {
     const int j1 = r % d1;
     const int j0 = r / d1;
     const int ia = ((j0 * s0) * D::g1 + j1 * s1) * D::g2 + j2 * s2;
-    haar2(s[ia], s[ia + off]);
+    haar2<S>(s[ia], s[ia + off]);
   }
   __syncthreads();
 }
 
-template <int J, int L>
+template <int J, int L, Scale S>
 __device__ __forceinline__ void haar_level(float2* s, bool inverse) {
   constexpr int st = 1 << (L - 2);  // level L >= 2 on the level-1 approximations
   if (!inverse) {
-    haar_pass<J, st, 0>(s);
-    haar_pass<J, st, 1>(s);
-    haar_pass<J, st, 2>(s);
+    haar_pass<J, st, 0, S>(s);
+    haar_pass<J, st, 1, S>(s);
+    haar_pass<J, st, 2, S>(s);
   } else {
-    haar_pass<J, st, 2>(s);
-    haar_pass<J, st, 1>(s);
-    haar_pass<J, st, 0>(s);
+    haar_pass<J, st, 2, S>(s);
+    haar_pass<J, st, 1, S>(s);
+    haar_pass<J, st, 0, S>(s);
   }
 }
 
 // Levels 2..J forward (inverse) on the shared approximations; callers
 // synchronise before the first pass.
-template <int J>
+template <int J, Scale S>
 __device__ void upper_forward(float2* s) {
-  if constexpr (J >= 2) haar_level<J, 2>(s, false);
-  if constexpr (J >= 3) haar_level<J, 3>(s, false);
-  if constexpr (J >= 4) haar_level<J, 4>(s, false);
+  if constexpr (J >= 2) haar_level<J, 2, S>(s, false);
+  if constexpr (J >= 3) haar_level<J, 3, S>(s, false);
+  if constexpr (J >= 4) haar_level<J, 4, S>(s, false);
 }
 
-template <int J>
+template <int J, Scale S>
 __device__ void upper_inverse(float2* s) {
-  if constexpr (J >= 4) haar_level<J, 4>(s, true);
-  if constexpr (J >= 3) haar_level<J, 3>(s, true);
-  if constexpr (J >= 2) haar_level<J, 2>(s, true);
+  if constexpr (J >= 4) haar_level<J, 4, S>(s, true);
+  if constexpr (J >= 3) haar_level<J, 3, S>(s, true);
+  if constexpr (J >= 2) haar_level<J, 2, S>(s, true);
+}
+
+// 2^(1.5 l), l = 0..4: the scale of level l's coefficients under Scale::kSum
+__device__ __forceinline__ float level_scale(int l) {
+  return l == 0 ? 1.0f : l == 1 ? 2.82842712f : l == 2 ? 8.0f : l == 3 ? 22.6274170f : 64.0f;
 }
 
 // In place: v <- W^H soft(W v, tau) for the group's eight values, levels
@@ -268,21 +285,28 @@ __device__ __forceinline__ void prox_group(float2 v[8], float2* s, float tau) {
 #pragma unroll
     for (int k = 0; k < 8; ++k) v[k] = soft(v[k], tau);
   } else {
-    haar8_forward(v);
+    haar8_forward<Scale::kSum>(v);
+    const float tau1 = tau * level_scale(1);
 #pragma unroll
-    for (int k = 1; k < 8; ++k) v[k] = soft(v[k], tau);
+    for (int k = 1; k < 8; ++k) v[k] = soft(v[k], tau1);
     if constexpr (J == 1) {
-      v[0] = soft(v[0], tau);
+      v[0] = soft(v[0], tau1);
     } else {
       s[threadIdx.x] = v[0];
       __syncthreads();
-      upper_forward<J>(s);
-      s[threadIdx.x] = soft(s[threadIdx.x], tau);
+      upper_forward<J, Scale::kSum>(s);
+      // the level of the thread's entry: a detail of level 2 + the trailing zeros that
+      // its group coordinates share, or the approximation of level J
+      using D = Box<J>;
+      const int t = threadIdx.x;
+      const int shared_zeros = __ffs(t % D::g2 | (t / D::g2) % D::g1 | t / (D::g2 * D::g1)) - 1;
+      const int level = shared_zeros < 0 ? J : min(J, 2 + shared_zeros);
+      s[threadIdx.x] = soft(s[threadIdx.x], tau * level_scale(level));
       __syncthreads();
-      upper_inverse<J>(s);
+      upper_inverse<J, Scale::kHalfSum>(s);
       v[0] = s[threadIdx.x];
     }
-    haar8_inverse(v);
+    haar8_inverse<Scale::kHalfSum>(v);
   }
 }
 
@@ -443,11 +467,11 @@ __global__ void __launch_bounds__(Box<J>::nt) wavelet_kernel(const float2* __res
     else
 #pragma unroll
       for (int k = 0; k < 8; ++k) v[k] = make_float2(0.0f, 0.0f);
-    if constexpr (J >= 1) haar8_forward(v);
+    if constexpr (J >= 1) haar8_forward<Scale::kOrthonormal>(v);
     if constexpr (J >= 2) {
       s[threadIdx.x] = v[0];
       __syncthreads();
-      upper_forward<J>(s);
+      upper_forward<J, Scale::kOrthonormal>(s);
       v[0] = s[threadIdx.x];
     }
     if (!gr.any) return;
@@ -468,10 +492,10 @@ __global__ void __launch_bounds__(Box<J>::nt) wavelet_kernel(const float2* __res
   if constexpr (J >= 2) {
     s[threadIdx.x] = v[0];
     __syncthreads();
-    upper_inverse<J>(s);
+    upper_inverse<J, Scale::kOrthonormal>(s);
     v[0] = s[threadIdx.x];
   }
-  if constexpr (J >= 1) haar8_inverse(v);
+  if constexpr (J >= 1) haar8_inverse<Scale::kOrthonormal>(v);
   if (gr.any) store8(out, g, gr, v);
 }
 
