@@ -586,20 +586,27 @@ __global__ void __launch_bounds__(32 * WPC, WPC == 4 ? 5 : 16 / WPC) spread_coil
 // fall by 29 %.  Rows m = 16 z + 4 y + x of the sub-block (z, y, x in 0..3):
 // lane (g, q) holds x = g % 4 with y = g / 4 (row g) and y + 2 (row g + 8) for
 // every m-tile z.  Columns and the TF32 split are those of the plane kernel.
-// EXACT (FP32 grids): every k-step's eight points are summed from a zero
-// accumulator, small terms first, and added to the sums by one rounded FP32
-// addition (16 more additions per k-step): the tensor core truncates its running
-// sum, which over a dense sub-block's hundreds of steps costs a few 1e-6, and
-// which a CG solve then carries on (64^3, 8 coils, six iterations: 2e-6 to 1e-5).
-// 256^3, 16 coils, 3 M samples: 4.20 (at 24 warps per SM; the whole adjoint 12.53 ->
-// 12.21 ms with 28) against 4.01 ms, error of the adjoint on
-// positive data 2.8e-7 against 5.3e-6 (register kernel 6.50 ms, 2.9e-7).  E at
-// 128^3, 8 coils, 4 phases: 8.18 against 8.15 ms (8.28 at 24 warps per SM).
+// Sums.  kRunning (BF16 grids): the tensor core's accumulator, which it truncates; over a
+// dense sub-block's hundreds of steps that costs a few 1e-6, which a CG solve then carries
+// on (64^3, 8 coils, six iterations: 2e-6 to 1e-5).  kSteps (FP32 grids, tuned plans): every
+// k-step's eight points are summed from a zero accumulator, small terms first, and added to
+// the sums by one rounded FP32 addition (16 more additions per k-step).  256^3, 16 coils,
+// 3 M samples: 4.20 (at 24 warps per SM; the whole adjoint 12.53 -> 12.21 ms with 28) against
+// 4.01 ms, error of the adjoint on positive data 2.8e-7 against 5.3e-6 (register kernel 6.50 ms,
+// 2.9e-7).  E at 128^3, 8 coils, 4 phases: 8.18 against 8.15 ms (8.28 at 24 warps per SM).
+// kHalves (untuned plans, which take this kernel without having asked for a tensor-core
+// one): the leading products of four points each from zero, all three parts joined by FP32
+// additions, as accurate as the register kernel.  Errors of E on 10 geometries with 3 sets of
+// inputs each against those of the register kernel, geometric mean: kSteps 1.066, kHalves
+// 0.972 (the leading products of eight points apart from the small terms 1.018; more of the
+// low parts no better).  The adjoint above 12.59 against 12.20 ms.
 // A k-step skips the m-tiles none of its eight points reaches (the runs are in
 // first-tap z order, so neighbouring points mostly share their z planes).  The
 // launch bound of 28 warps per SM holds the W = 4 kernel at 72 registers; with one
 // warp per CTA (the usual choice) a CTA's slot frees as soon as its sub-block
 // is done, whatever the other sub-blocks' point counts.
+enum class CubeSum { kRunning, kSteps, kHalves };
+
 template <int W>
 struct CubeStage {
   static constexpr int PW = (W + 3) / 4 * 4;
@@ -617,7 +624,7 @@ __device__ __forceinline__ void put_taps(float* dst, const float (&w)[W]) {
   if constexpr (W == 6) reinterpret_cast<float2*>(dst)[2] = make_float2(w[4], w[5]);
 }
 
-template <typename GT, int WPC, int W, bool EXACT>
+template <typename GT, int WPC, int W, CubeSum SUM>
 __global__ void __launch_bounds__(32 * WPC, (W == 6 ? 24 : 28) / WPC) spread_coils_cube_kernel(
     Geo g, KernelCoefs kc, int C, TilePlan tp, PhaseTable pt, const float2* __restrict__ vals,
     GT* __restrict__ grids, float2* __restrict__ scratch) {
@@ -774,13 +781,21 @@ __global__ void __launch_bounds__(32 * WPC, (W == 6 ? 24 : 28) / WPC) spread_coi
           split_tf32(a[1][1], ah[3], al[3]);
 #pragma unroll
           for (int nt = 0; nt < 2; ++nt) {
-            if constexpr (EXACT) {
+            if constexpr (SUM != CubeSum::kRunning) {
               float d[4];
               mma_tf32_zero(d, al[0], al[1], al[2], al[3], bh[nt][0], bh[nt][1]);
               mma_tf32(d, ah[0], ah[1], ah[2], ah[3], bl[nt][0], bl[nt][1]);
-              mma_tf32(d, ah[0], ah[1], ah[2], ah[3], bh[nt][0], bh[nt][1]);
+              if constexpr (SUM == CubeSum::kHalves) {
+                float d0[4], d1[4];
+                mma_tf32_half(d0, ah[0], ah[1], bh[nt][0]);
+                mma_tf32_half(d1, ah[2], ah[3], bh[nt][1]);
 #pragma unroll
-              for (int i = 0; i < 4; ++i) acc[mt][nt][i] += d[i];
+                for (int i = 0; i < 4; ++i) acc[mt][nt][i] += (d0[i] + d1[i]) + d[i];
+              } else {
+                mma_tf32(d, ah[0], ah[1], ah[2], ah[3], bh[nt][0], bh[nt][1]);
+#pragma unroll
+                for (int i = 0; i < 4; ++i) acc[mt][nt][i] += d[i];
+              }
             } else {
               mma_tf32(acc[mt][nt], ah[0], ah[1], ah[2], ah[3], bh[nt][0], bh[nt][1]);
               mma_tf32(acc[mt][nt], ah[0], ah[1], ah[2], ah[3], bl[nt][0], bl[nt][1]);
@@ -1261,27 +1276,36 @@ int launch_reduce(const Geo& g, int C, const TilePlan& tp, const PhaseTable& pt,
 }
 
 // the sub-block spread over 8-coil chunks, wpc (1, 2 or 4) sub-blocks per CTA; BF16
-// grids keep the tensor core's running sum, whose error their rounding covers
+// grids keep the tensor core's running sum, whose error their rounding covers; halves: the
+// sums of the register kernel's accuracy (W = 4; at W = 6 the alternative is the generic
+// kernel, whose error is the larger one)
 template <typename GT, int W>
 void launch_cube(const Geo& g, const KernelCoefs& kc, int C, const TilePlan& tp,
                  const PhaseTable& pt, const float2* vals, GT* grids, float2* scratch, int wpc,
-                 cudaStream_t s) {
-  constexpr bool kExact = sizeof(GT) == 8;
+                 bool halves, cudaStream_t s) {
+  constexpr CubeSum kSum = sizeof(GT) == 8 ? CubeSum::kSteps : CubeSum::kRunning;
   const unsigned blocks = 8u * pt.item0[pt.nphase];
   const int chunks = (C + 7) / 8;
-  if constexpr (W == 4) {
-    if (wpc == 4) {
-      spread_coils_cube_kernel<GT, 4, W, kExact><<<dim3(blocks / 4, chunks), 128, 0, s>>>(
-          g, kc, C, tp, pt, vals, grids, scratch);
-      return;
-    }
-    if (wpc == 2) {
-      spread_coils_cube_kernel<GT, 2, W, kExact><<<dim3(blocks / 2, chunks), 64, 0, s>>>(
+  if constexpr (W == 4 && sizeof(GT) == 8) {
+    if (halves) {
+      spread_coils_cube_kernel<GT, 1, W, CubeSum::kHalves><<<dim3(blocks, chunks), 32, 0, s>>>(
           g, kc, C, tp, pt, vals, grids, scratch);
       return;
     }
   }
-  spread_coils_cube_kernel<GT, 1, W, kExact><<<dim3(blocks, chunks), 32, 0, s>>>(
+  if constexpr (W == 4) {
+    if (wpc == 4) {
+      spread_coils_cube_kernel<GT, 4, W, kSum><<<dim3(blocks / 4, chunks), 128, 0, s>>>(
+          g, kc, C, tp, pt, vals, grids, scratch);
+      return;
+    }
+    if (wpc == 2) {
+      spread_coils_cube_kernel<GT, 2, W, kSum><<<dim3(blocks / 2, chunks), 64, 0, s>>>(
+          g, kc, C, tp, pt, vals, grids, scratch);
+      return;
+    }
+  }
+  spread_coils_cube_kernel<GT, 1, W, kSum><<<dim3(blocks, chunks), 32, 0, s>>>(
       g, kc, C, tp, pt, vals, grids, scratch);
 }
 
@@ -1341,7 +1365,8 @@ int dispatch_coils(const Geo& g, const KernelCoefs& kc, int C, const TilePlan& t
     if constexpr (CC < 8 && sizeof(GT) == 8) launch_few<CC, 4>(g, kc, C, tp, pt, vals, grids, scratch, s);
   } else if (CC == 8 && ((variant == kSpreadMMA && mma_cube) || variant == kSpreadCubeExact) &&
              pt.clist[0] != nullptr) {
-    launch_cube<GT, 4>(g, kc, C, tp, pt, vals, grids, scratch, mma_wpc, s);
+    launch_cube<GT, 4>(g, kc, C, tp, pt, vals, grids, scratch, mma_wpc,
+                       variant == kSpreadCubeExact, s);
   } else if (variant == kSpreadMMA && CC == 8) {
     const unsigned planes = 8u * pt.item0[pt.nphase];
     if (mma_wpc == 4)
@@ -1403,7 +1428,7 @@ int spread_multi(const Geo& g, int W, const KernelCoefs& kc, int C, const TilePl
         launch_few<4, 6>(g, kc, C, tp, pt, v, gr, sc, s);
         return 1 + launch_reduce<8, 4, GT>(g, C, tp, pt, chunks, gr, sc, s);
       }
-      launch_cube<GT, 6>(g, kc, C, tp, pt, v, gr, sc, 1, s);
+      launch_cube<GT, 6>(g, kc, C, tp, pt, v, gr, sc, 1, false, s);
       return 1 + launch_reduce<8, 8, GT>(g, C, tp, pt, chunks, gr, sc, s);
     }
   }

@@ -1061,10 +1061,9 @@ nrsense_status create_impl(nrsense_plan_s* p, const nrsense_desc* desc, const in
     // launch choices until the plan is tuned.  Interpolation from TMA-staged halos
     // of 4 coils (bitwise the per-value staging's results; 1.60 against 2.97 ms
     // at 128^3, 8 coils, 4 phases; the tuned choice there).  FP32 spread by
-    // sub-blocks with FP32-accurate sums: on the tensor cores, eight points per
-    // rounded addition (5 to 8 coils and chunks of 8; 256^3, 16 coils, 3 M
-    // samples: below 4.20 ms against 6.50 of the register kernel, the adjoint's error
-    // 2.6e-7 against 2.7e-7), or by FMAs (1 and 2 coils, where that is the faster one:
+    // sub-blocks: on the tensor cores with sums of the register kernel's accuracy
+    // (CubeSum::kHalves; 5 to 8 coils and chunks of 8; 256^3, 16 coils, 3 M samples: below
+    // 4.5 ms against 6.50 of the register kernel), or by FMAs (1 and 2 coils, where that is the faster one:
     // few_pays, kernels_spread.cu; with 3 and 4 coils the register kernel is the faster
     // one on dense samples, 0.495 against 0.634 ms at 128^3, and the tuner times both).
     // BF16 grids keep the register kernel and its exact summation order.
