@@ -560,7 +560,7 @@ nrsense_status nrsense_symmetric_eigen(int32_t m, const double* a_host, double* 
 #define NRSENSE_TUNE_SPREAD_MMA           4  /* tensor-core accumulation (TF32 split in three
                                                 products), a warp per tile plane or per 4^3
                                                 sub-block, 8-coil chunks
-                                                (four coils and fewer: FP32 FMAs by sub-blocks;
+                                                (two to four coils: FP32 FMAs by sub-blocks;
                                                 BF16 grids: as REGISTER_WARP); within FP32
                                                 rounding of, not bitwise equal to, the others */
 typedef struct {
@@ -575,15 +575,20 @@ typedef struct {
                                   (both over per-tile halo lists), 2 home tiles (every displaced
                                   voxel spread once by the warp of the 8^3 tile holding its first
                                   tap, super-tile rims summed by a second kernel; on grids with
-                                  at most a point per six values, rows of 4^3 blocks instead;
+                                  at most a point per six values, not crowded into a few rows,
+                                  rows of 4^3 blocks instead;
                                   W = 4 and not compensated; set_tuning rejects 2 elsewhere) */
   double  spread_image_ms[3];  /* measured: CTA per tile, CTA per plane pair, home tiles
                                   (-1: n/a) */
   int32_t fft_pruned;          /* 1: own pruned coil-grid transforms with the coil fan-out and
                                   combination fused (sigma 2, power-of-two grid sizes 32..256,
-                                  FP32 grids); 0: cuFFT plus the fan-out / combination kernels
-                                  (grids of other sizes take the mixed-radix passes either way,
-                                  where their prime factors are at most 13) */
+                                  FP32 grids; with 128 points along axes 0 and 1 these are the
+                                  mixed-radix passes); 0: cuFFT plus the fan-out / combination
+                                  kernels (grids of other sizes take the mixed-radix passes
+                                  either way where every axis has them: G = 2 N with N = R S, R
+                                  even, R and S at most 16, or N and G each a product r1 r2 r3
+                                  with r1 and r3 in 2..16 and r2 in 1..8; of 1024 points along
+                                  axis 0 and 1024 along axis 1 or 896 along axis 2, cuFFT) */
   double  fft_ms[2];           /* measured forward + adjoint of the first phase chunk:
                                   cuFFT path, pruned path (-1: not available) */
   double  spread_mma_ms;       /* measured tensor-core spread, best geometry and warps per CTA
@@ -614,7 +619,7 @@ typedef struct {
                                   power-of-two grid sizes 32..256, not with the compensated
                                   precision; set_tuning rejects 1 elsewhere), 0 cuFFT plus the
                                   deapodization kernels (grids of other sizes: the mixed-radix
-                                  passes either way, as above) */
+                                  passes either way, where every axis has them) */
   double  image_fft_ms[2];     /* measured forward + adjoint G^3 transforms with their
                                   deapodization: cuFFT path, pruned path (-1: n/a) */
 } nrsense_tuning;

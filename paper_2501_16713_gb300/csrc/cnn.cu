@@ -526,7 +526,7 @@ __global__ void __launch_bounds__(kTcThreads, 4) conv3d_tc_kernel(
 // with one CTA of 12 warps per SM (the 72 accumulators): the copies of the next
 // block run under the products of this one (2 x 76 KB of stages).  Two pairs of
 // 128^3, twelve calls: with the parallel reduction below 9.95 -> 8.24 ms for the
-// whole gradient and application, the sums bit for bit as before.
+// whole gradient and application; the partial sums bit for bit as before.
 __global__ void __launch_bounds__(kWgThreads, 1) wgrad_kernel(Vol v, const bf16* __restrict__ in,
                                                                const bf16* __restrict__ gr,
                                                                float* __restrict__ part_w,

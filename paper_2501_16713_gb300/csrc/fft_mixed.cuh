@@ -13,12 +13,12 @@
 // computed: a radix-2R butterfly with R nonzero inputs is two radix-R ones
 // (even outputs of v, odd outputs of v W_2R^n), with R wanted outputs two
 // radix-R ones of the even and the odd inputs.  One exchange through shared
-// memory per transform.  The radices are template values for the axis lengths
-// of the common volumes (strides, masks and twiddle indices become constants)
-// and run-time values, with one unrolled body per radix behind a CTA-uniform
+// memory per transform.  The radices are template values for N a multiple of 16 up
+// to 256 (strides, masks and twiddle indices become constants) and run-time values, with one unrolled body per radix behind a CTA-uniform
 // switch, for the rest.
-// GeneralAxis (any G <= 1024 with prime factors up to 13): in place, decimation
-// in frequency, two or three steps of radix 2..16.
+// GeneralAxis (N and G each r1 r2 r3 with r1 and r3 in 2..16 and r2 in 1..8: of the
+// lengths of 16 to 1024 without a prime above 13 all but 625, 729, 875, 891, 972 and
+// 1000): in place, decimation in frequency, two or three steps.
 #pragma once
 
 #include <type_traits>

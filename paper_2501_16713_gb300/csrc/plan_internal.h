@@ -31,7 +31,7 @@ struct PointSet {
   int2* list = nullptr;
   SpreadItem* items = nullptr;  // heaviest first
   int32_t* bins = nullptr;      // per item: W + T + 1 plane-offset bin starts (relative)
-  // 8^3 tiles, W = 4: the list with every item's entries ordered by footprint
+  // 8^3 tiles: the list with every item's entries ordered by footprint
   // class (4^3 sub-blocks touched), and kCubeBins class starts per item
   int2* clist = nullptr;
   int32_t* cbins = nullptr;
@@ -49,6 +49,10 @@ struct PointSet {
 }  // namespace nrs
 
 namespace nrs {
+// Spread variants (launch_spread, launch_spread_home / _rows).
+constexpr int kSpreadRegister = 1, kSpreadShared = 2, kSpreadRegisterWarp = 3, kSpreadMMA = 4,
+              kSpreadHome = 5, kSpreadCubeExact = 6;
+
 // One transform length of the mixed-radix passes (fft_mixed.cuh): L = r1 r2 r3,
 // s = r2 r3, ceil(2^32 / d) of the divisors d its index arithmetic needs.
 struct MixLen {
@@ -190,7 +194,7 @@ struct nrsense_plan_s {
   // is the generic halo-list kernel), for W = 4 as the kSpreadHome choice of
   // sparse plans
   bool spread_rows() const {
-    return rows_ok && (W != 4 || (rows_sparse && spread_image_variant == 5));
+    return rows_ok && (W != 4 || (rows_sparse && spread_image_variant == nrs::kSpreadHome));
   }
   bool own_image_fft() const { return image_fft_pruned || (image_mixed && !image_fft_ok); }
   bool pad_dirty = false;      // b_xpad / b_xmid hold the pruned transforms' intermediates
@@ -318,8 +322,6 @@ int launch_crop_to_coils(const Geo& g, int C, const float* deapod, const void* x
 // compensated accumulation (W = 4 kernels); variant selects register or
 // shared-memory accumulation for the multi-coil W = 4 kernel (register
 // accumulation with a CTA per tile, or with a CTA per tile plane).
-constexpr int kSpreadRegister = 1, kSpreadShared = 2, kSpreadRegisterWarp = 3, kSpreadMMA = 4,
-              kSpreadHome = 5, kSpreadCubeExact = 6;
 // a spread variant value carries, in bits 8-15, the warps per CTA of the
 // tensor-core kernel (1, 2 or 4; 0 means 1) and, in bit 16, its geometry
 // (0: a warp per tile plane, 1: a warp per 4^3 sub-block)
@@ -344,7 +346,7 @@ long long home_scratch_elems(const HomeSet& hs);
 // largest number of points a warp of the row spread visits, into *most (zeroed
 // before; spread_rows.cu)
 int launch_row_load(int W, const RowSet& rs, int32_t* most, cudaStream_t s);
-// row spread on the tensor cores (spread_rows.cu): all points of `rs` into grid
+// row spread (FP32 FMAs, spread_rows.cu): all points of `rs` into grid
 int launch_spread_rows(const Geo& g, int W, const KernelCoefs& kc, const RowSet& rs,
                        const nrsense_c64* vals, nrsense_c64* grid, cudaStream_t s);
 // image-space interpolation over the same super-tiles (spread_home.cu): m rows
