@@ -63,7 +63,10 @@ def _set(plan, **kw):
 def test_image_interpolation(shape, osf, phases):
     import torch
     from paper_2501_16713_gb300 import Plan
-    plan = Plan(shape, disp=to_dev(_contraction(shape, phases, 0.95)), n_phases=phases, osf=osf)
+    size = max(shape)  # motion as in the benchmark: bumps of up to 6 % of the image
+    d = np.stack([synth.bump_displacement(shape, 169 + j, 0.06 * size, width_range=(0.05 * size, 0.1 * size))
+                  for j in range(phases)])
+    plan = Plan(shape, disp=to_dev(d), n_phases=phases, osf=osf)
     x = to_dev(crandn(np.random.default_rng(161), shape))
     out = plan.warp_forward(x)
     run = lambda: plan.warp_forward(x, out=out)  # noqa: E731
