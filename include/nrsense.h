@@ -549,8 +549,9 @@ nrsense_status nrsense_symmetric_eigen(int32_t m, const double* a_host, double* 
  * space; plans without coils tune only the image-space spread.
  * nrsense_plan_set_tuning applies stored choices (e.g. a cache keyed by the
  * geometry).  Both change only speed: every choice computes the same values
- * (bitwise, except the tensor-core spread and the pruned transforms, which
- * agree to FP32 rounding).  set_tuning builds the image-space point order that a choice
+ * (bitwise, except the tensor-core and sub-block spreads, the point orders
+ * of the image-space spread and the own transforms, which agree to FP32 rounding, and the
+ * last bit of image-space interpolations whose displacement is a negative below 1e-7).  set_tuning builds the image-space point order that a choice
  * needs where the plan does not have it yet (device memory; synchronises).
  * Errors: ERR_ARG (null, reps outside 1..100, unknown choice), ERR_CUDA.
  */

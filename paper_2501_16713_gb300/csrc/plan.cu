@@ -838,7 +838,8 @@ nrsense_status create_impl(nrsense_plan_s* p, const nrsense_desc* desc, const in
     if (rows && (p->W != 4 || 6 * p->P * g.nvox <= g.ngrid)) NRS_TRY(build_row_set(p, s));
     p->rows_sparse = p->rows_ok && p->W == 4;
     if (!p->rows_ok) NRS_TRY(p->home_ok ? build_home_set(p, s) : build_image_lists(p, s));
-    // Interpolation until the plan is tuned (bitwise the same values): a thread per
+    // Interpolation until the plan is tuned (the same values, but for the last bit where a
+    // negative displacement below 1e-7 rounds up to the grid point in FP64): a thread per
     // voxel, or from super-tiles staged in shared memory.  Per voxel at sigma 2: 0.324
     // against 0.429 ms at 192^3 with one phase, 0.302 against 0.311 at 128^3 with four;
     // but 0.571 against 0.480 with eight (0.248 against 0.202 at 96^3, equal at 64^3).

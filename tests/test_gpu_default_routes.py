@@ -72,11 +72,17 @@ def test_image_interpolation(shape, osf, phases):
     run = lambda: plan.warp_forward(x, out=out)  # noqa: E731
     ms, first = _stage(plan, "interp_image", run), out.clone()
     other = []
+    dt = to_dev(d)
+    edge = ((dt < 0) & (dt > -1e-7)).any(1)
     own = int(osf == 2 and set(shape) <= {16, 32, 64, 128})  # power-of-two transforms, as created
     for home in (0, 1):
         _set(plan, interp_image_home=home, spread_image_warp=2, image_fft_pruned=own)
         other.append(_stage(plan, "interp_image", run))
-        assert torch.equal(out, first)
+        # the same values, bit for bit but where a displacement component is negative and
+        # below 1e-7: the sorted positions (FP64) round up to the grid point, whose taps
+        # start one later with the fraction 0 instead of 1
+        same = (out == first) | edge
+        assert bool(same.all()) and float((out - first).abs().max()) < 1e-6 * float(first.abs().max())
     print(shape, osf, phases, "default %.4f, per voxel %.4f, super-tiles %.4f ms" % (ms, *other))
     assert ms < 1.1 * min(other)
     plan.close()
