@@ -551,8 +551,9 @@ nrsense_status nrsense_symmetric_eigen(int32_t m, const double* a_host, double* 
  * geometry).  Both change only speed: every choice computes the same values
  * (bitwise, except the tensor-core and sub-block spreads, the point orders
  * of the image-space spread and the own transforms, which agree to FP32 rounding, and the
- * last bit of image-space interpolations whose displacement is a negative below 1e-7).  set_tuning builds the image-space point order that a choice
- * needs where the plan does not have it yet (device memory; synchronises).
+ * last bit of image-space interpolations whose displacement is a negative below
+ * 1e-7).  set_tuning builds the image-space point order that a choice needs where the
+ * plan does not have it yet (device memory; synchronises).
  * Errors: ERR_ARG (null, reps outside 1..100, unknown choice), ERR_CUDA.
  */
 #define NRSENSE_TUNE_SPREAD_REGISTER      1  /* register accumulation, CTA per tile */

@@ -842,7 +842,8 @@ nrsense_status create_impl(nrsense_plan_s* p, const nrsense_desc* desc, const in
     // negative displacement below 1e-7 rounds up to the grid point in FP64): a thread per
     // voxel, or from super-tiles staged in shared memory.  Per voxel at sigma 2: 0.324
     // against 0.429 ms at 192^3 with one phase, 0.302 against 0.311 at 128^3 with four;
-    // but 0.571 against 0.480 with eight (0.248 against 0.202 at 96^3, equal at 64^3).
+    // but 0.571 against 0.480 with eight (0.248 against 0.202 at 96^3, equal at 64^3; without
+    // the rigid shifts that part the phases' taps 0.542 against 0.563).
     // A rational sigma decomposes every position in FP64, which the super-tiles' sorted
     // points hold ready: 0.387 against 0.101 ms at 128^3, sigma 1.5; with no more CTAs
     // than SMs that hides (0.014 against 0.020 ms at 32^3; 0.030 against 0.019 at 48^3).
